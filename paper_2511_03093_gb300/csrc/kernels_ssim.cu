@@ -186,8 +186,9 @@ cslsm_status launch_ssim3d(const float *x, const float *ref, int Z, int H, int W
     cslsm_status st = set_weights(dev);
     if (st) return st;
     const size_t N = (size_t)Z * H * W;
-    float *fields = (float *)ws;
-    double *partials = (double *)(fields + 5 * N);
+    // the FP64 partials first: behind the fields they would be misaligned for odd N
+    double *partials = (double *)ws;
+    float *fields = (float *)(partials + nblocks);
     {
         LaunchScope ls(K_SSIM, s);
         const dim3 grid((W + kTX - 1) / kTX, (H + kTY - 1) / kTY, Z);

@@ -46,6 +46,15 @@ def test_matches_oracle(cs, shape):
     assert abs(got - ref) <= BAR, (got, ref)
 
 
+@pytest.mark.parametrize("shape", [(3, 5, 7), (1, 63, 65), (21, 41, 39)])
+def test_odd_voxel_count(cs, shape):
+    """The FP64 partial sums stay aligned when Z * H * W is odd."""
+    x, y = _pair(sum(shape), shape)
+    got = float(cs.ssim3d(to_dev(y), to_dev(x)))
+    ref = oracle.ssim3d(y, x)
+    assert abs(got - ref) <= BAR, (got, ref)
+
+
 def test_identical_volumes(cs):
     x, _ = _pair(5, (9, 40, 70))
     assert abs(float(cs.ssim3d(to_dev(x), to_dev(x))) - 1.0) <= 1e-6
