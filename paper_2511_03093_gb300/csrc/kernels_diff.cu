@@ -27,10 +27,8 @@
 // iterates and runs their adjoint), the x-update.  Gradients: dL/dlogits and
 // the three scalars dL/drho, dL/dlambda, dL/dgamma (FP64 accumulators).
 //
-// Kernels are one-thread-per-pixel passes (a block row of the grid per batch
-// item); the stencils read their neighbours from global memory (L1/L2), except
-// that the forward dual step forms q once per tile in shared memory and the
-// reverse dual step works on shared-memory tiles.
+// The x-update kernels are one-thread-per-pixel passes (a block row of the grid
+// per batch item); the u-step runs several dual steps per launch on chip (below).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -39,6 +37,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "tv_body.cuh"
 
 namespace cslsm {
 namespace {
@@ -49,20 +48,40 @@ constexpr int kT = 256;
 // one address per scalar would serialise tens of thousands of atomics a launch.
 constexpr int kAccCopies = 64;
 
-// Adds the block's sum of v to acc[idx][blockIdx.x % kAccCopies].  Every thread
-// of the block must call it.
-__device__ __forceinline__ void block_acc(double v, double *acc, int idx)
+// A sum kept as an unevaluated pair of FP32 numbers (Knuth's two-sum): about 48
+// bits, at FP32 rates.  An FP64 addition occupies an SM for 16 cycles a warp
+// here, so FP64 block sums took as long as the reverse steps they followed.
+struct Pair32 {
+    float hi, lo;
+    __device__ __forceinline__ void add(float h, float l)
+    {
+        const float s = hi + h, v = s - hi;
+        lo += ((hi - (s - v)) + (h - v)) + l;
+        hi = s;
+    }
+};
+
+// Adds the block's sums of v[0 .. N) to acc[idx[.]][blockIdx.x % kAccCopies].
+// Every thread of the block must call it.
+template <int N>
+__device__ __forceinline__ void block_acc(Pair32 (&v)[N], double *acc, const int (&idx)[N])
 {
-    __shared__ double s_part[kT / 32];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kT / 32; ++w) t += s_part[w];
-        atomicAdd(acc + idx * kAccCopies + blockIdx.x % kAccCopies, t);
+    __shared__ Pair32 s_part[N][32];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        for (int off = 16; off > 0; off >>= 1)
+            v[q].add(__shfl_down_sync(0xffffffffu, v[q].hi, off),
+                     __shfl_down_sync(0xffffffffu, v[q].lo, off));
+        if ((threadIdx.x & 31) == 0) s_part[q][threadIdx.x >> 5] = v[q];
     }
     __syncthreads();
+    if (threadIdx.x < N) {
+        Pair32 t = s_part[threadIdx.x][0];
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+            t.add(s_part[threadIdx.x][w].hi, s_part[threadIdx.x][w].lo);
+        atomicAdd(acc + idx[threadIdx.x] * kAccCopies + blockIdx.x % kAccCopies,
+                  (double)t.hi + (double)t.lo);
+    }
 }
 
 struct Geo {
@@ -72,16 +91,6 @@ struct Geo {
 };
 
 __device__ __forceinline__ float sigm(float x) { return 1.f / (1.f + expf(-x)); }
-
-// div of a dual field (components along rows p1, along columns p2) with the
-// Neumann boundary of the forward differences.
-__device__ __forceinline__ float divp(const float *p1, const float *p2, int i, int j, int H, int W)
-{
-    const size_t o = (size_t)i * W + j;
-    const float a = (i < H - 1 ? p1[o] : 0.f) - (i > 0 ? p1[o - W] : 0.f);
-    const float c = (j < W - 1 ? p2[o] : 0.f) - (j > 0 ? p2[o - 1] : 0.f);
-    return a + c;
-}
 
 // ---- x-update ----------------------------------------------------------------
 __global__ void ux_fwd_kernel(const float *__restrict__ U, const float *__restrict__ Dl,
@@ -121,7 +130,7 @@ __global__ void ux_bwd_kernel(const float *__restrict__ U, const float *__restri
 {
     const size_t p = blockIdx.x * (size_t)kT + threadIdx.x;
     const int bi = blockIdx.y;
-    double rho_bar = 0.0;
+    Pair32 rho_bar[1] = {};
     if (p < g.HW()) {
         const size_t base = bi * g.NV() + p, HW = g.HW();
         float s = 0.f, D = 0.f, ebar = 0.f;
@@ -137,7 +146,7 @@ __global__ void ux_bwd_kernel(const float *__restrict__ U, const float *__restri
         const float e = (b[bi * HW + p] - s) / den;
         const float sbar = -ebar / den;
         const float Dbarv = -ebar * e / den;
-        rho_bar = (double)(-ebar * e / den);
+        rho_bar[0].hi = -ebar * e / den;
         for (int r = 0; r < g.Z; ++r) {
             const size_t o = base + r * HW;
             const float m = sigm(logits[o]);
@@ -150,271 +159,594 @@ __global__ void ux_bwd_kernel(const float *__restrict__ U, const float *__restri
             lbar[o] += mbar * m * (1.f - m);
         }
     }
-    block_acc(rho_bar, acc, 0);
+    const int idx[1] = {0};
+    block_acc(rho_bar, acc, idx);
 }
 
-// ---- u-step: g formation -----------------------------------------------------
-// h = (rho w_n + gamma (A + C)) / (rho + 2 gamma), A, C the neighbour slices.
-__global__ void hform_kernel(const float *__restrict__ Wn, const float *A, const float *C, Geo g,
-                             float rho, float gam,
-                             float *__restrict__ Hb)
-{
-    const size_t p = blockIdx.x * (size_t)kT + threadIdx.x;
-    const int bi = blockIdx.y;
-    if (p >= g.HW()) return;
-    const size_t o = bi * g.NV() + p;
-    const float s = gam > 0.f ? A[o] + C[o] : 0.f;
-    Hb[bi * g.HW() + p] = (rho * Wn[o] + gam * s) / (rho + 2.f * gam);
-}
-
-// Reverse of hform: hbar -> w_n, neighbours; direct dL/drho, dL/dgamma.
-__global__ void hform_bwd_kernel(const float *__restrict__ Hbar, const float *__restrict__ Wn,
-                                 const float *A, const float *C, Geo g,
-                                 float rho, float gam, float *__restrict__ Wn_bar,
-                                 float *A_bar, float *C_bar,  // may be the same slice (Z = 2)
-                                 double *__restrict__ acc)
-{
-    const size_t p = blockIdx.x * (size_t)kT + threadIdx.x;
-    const int bi = blockIdx.y;
-    double rb = 0.0, gb = 0.0;
-    if (p < g.HW()) {
-        const size_t o = bi * g.NV() + p;
-        const float den = rho + 2.f * gam;
-        const float hb = Hbar[bi * g.HW() + p];
-        const float s = gam > 0.f ? A[o] + C[o] : 0.f;
-        const float h = (rho * Wn[o] + gam * s) / den;
-        Wn_bar[o] += rho / den * hb;
-        if (gam > 0.f) {
-            A_bar[o] += gam / den * hb;
-            C_bar[o] += gam / den * hb;
-            gb = (double)(hb * (s - 2.f * h) / den);
-        }
-        rb = (double)(hb * (Wn[o] - h) / den);
-    }
-    block_acc(rb, acc, 0);
-    block_acc(gb, acc, 1);
-}
-
-// ---- Huber-TV prox: dual projected gradient ----------------------------------
-// q at (i, j) from p (both components, [bi] planes) and h.
-__device__ __forceinline__ float qval(const float *p1, const float *p2, const float *h, int i,
-                                      int j, int H, int W, float inv_theta)
-{
-    return divp(p1, p2, i, j, H, W) - h[(size_t)i * W + j] * inv_theta;
-}
-
-struct DualArgs {
-    const float *P;  // [B][2][H][W] p^t
-    float *Pn;       // [B][2][H][W] p^{t+1}
-    const float *Hb; // [B][H][W]
+// ---- u-step: the Huber-TV prox of one slice of every batch item ----------------
+// k dual steps per launch.  A CTA owns a TH x TW tile of one item's slice and
+// works on a region of NW RPW + 2 rows x 64 columns around it (halo of k + 1
+// rows, an even column halo): a warp holds RPW rows in registers, a lane two
+// adjacent columns, and only the warps' boundary rows go through shared memory,
+// one barrier a step.  Rows and columns of the halo go stale by one a step;
+// warps whose rows no later step needs skip.  One launch per dual step, h and u
+// apart, was bound by its 23 launches a slice (3.9 us each at 256 x 256) and at 8 x
+// 512 x 512 by its passes over memory; now the forward is bound by issue (67 % of
+// the slots, 43 us for 7 steps of 8 x 512 x 512), the reverse too (73 %, 86 us for
+// 5), and one small slice by the latency of a step and of a launch.  Forward +
+// backward, 10 iterations: 16 x 256 x 256 75.8 -> 17.8 ms; 8 x 16 x 512 x 512 with
+// the duals kept 242.5 -> 116.7 ms.
+//
+//   forward  first phase: h = (rho w_n + gamma (u_{n-1} + u_{n+1})) / (rho + 2
+//            gamma) on the region (kept for the later phases and the reverse
+//            pass), p = 0; each step q = div p - h / theta, a = p + tau (grad q -
+//            kappa p), p = a / max(1, |a|); last phase: u_n = h - theta div p,
+//            d_n = w_n - u_n.  With `rec` the a of every step is recorded (in place
+//            of the dual iterates, which a / max(1, |a|) gives back exactly).
+//   reverse  p^{t+1} = proj(a) with a recorded, so the Jacobian of the projection
+//            is local: abar = J(a)^T pbar^{t+1}, J = (I - a a^T / |a|^2) / |a|
+//            where |a| > 1; then qbar = -tau div abar and pbar^t = (1 - tau
+//            kappa) abar - grad qbar, the forward step's stencil once more.
+//            hbar = ubar - sum_t qbar / theta.  First phase: pbar^T = theta grad
+//            ubar; last phase: hbar to w_n, the neighbour slices and the scalars.
+//
+// The masks (0 on the last row / column and outside the image) keep p1 = 0 on
+// the last row and p2 = 0 on the last column, so div needs no boundary cases.
+struct HuberArgs {
+    const float *Wn, *A, *C;  // w_n and the neighbour slices, items N_V floats apart
+    float *Hb;                // [B][H][W] h
+    const float *Pin;         // [B][2][H][W] p (forward) / pbar (reverse) of the last
+    float *Pout;              //   phase or null; p / pbar for the next phase or null
+    float *rec;               // a of step t: rec + t [B][2][H][W], or null (forward)
+    float *Un, *Dn;           // forward, last phase: u_n and d_n (Un null: not wanted)
+    const float *Ubar;        // reverse: dL/du_n, items N_V floats apart
+    float *Hbar;              // reverse: [B][H][W]
+    float *Wbar, *Abar, *Cbar;  // reverse, last phase (Abar may be Cbar: Z = 2)
+    double *acc;
     Geo g;
-    float inv_theta, tau, kappa;
+    float rho, gam, theta, inv_theta, tau, kappa, eps;
+    int t0, ns;  // steps t0 .. t0 + ns - 1 (reverse: downwards)
+    int T;
+    int hh, hc, TH, TW, tx;
+    int pair;  // W even and the buffers 8-byte aligned: a lane's columns in one access
 };
 
-// One step p <- proj(p + tau (grad q - kappa p)) on a 2-D grid: blocks of 32
-// columns x 8 rows (row chunks grid-strided), z = batch item.  q is formed once
-// per pixel of the chunk, plus the row below and the column to the right that
-// grad q reads, into shared memory (by qval, as everywhere, so the same bits),
-// instead of three times per pixel.
-__global__ void __launch_bounds__(kT) dual_fwd_kernel(const DualArgs A)
+__device__ __forceinline__ float2 ld_pair(const float *p, int off, bool in0, bool in1, int pair)
 {
-    constexpr int R = kT / 32;  // rows per chunk
-    __shared__ float s_q[R + 1][33];
-    const Geo &g = A.g;
-    const int lane = (int)(threadIdx.x & 31), wr = (int)(threadIdx.x >> 5);
-    const int j0 = (int)blockIdx.x * 32, j = j0 + lane;
-    const int bi = blockIdx.z;
-    const float *p1 = A.P + (size_t)bi * 2 * g.HW(), *p2 = p1 + g.HW();
-    const float *h = A.Hb + (size_t)bi * g.HW();
-    float *n1 = A.Pn + (size_t)bi * 2 * g.HW(), *n2 = n1 + g.HW();
-    for (int i0 = (int)blockIdx.y * R; i0 < g.H; i0 += (int)gridDim.y * R) {
-        for (int t = (int)threadIdx.x; t < (R + 1) * 33; t += kT) {
-            const int r = t / 33, c = t - r * 33;
-            const int qi = i0 + r, qj = j0 + c;
-            if (qi < g.H && qj < g.W) s_q[r][c] = qval(p1, p2, h, qi, qj, g.H, g.W, A.inv_theta);
-        }
-        __syncthreads();
-        const int i = i0 + wr;
-        if (i < g.H && j < g.W) {
-            const float qc = s_q[wr][lane];
-            const float gx = i < g.H - 1 ? s_q[wr + 1][lane] - qc : 0.f;
-            const float gy = j < g.W - 1 ? s_q[wr][lane + 1] - qc : 0.f;
-            const size_t o = (size_t)i * g.W + j;
-            const float a1 = p1[o] + A.tau * (gx - A.kappa * p1[o]);
-            const float a2 = p2[o] + A.tau * (gy - A.kappa * p2[o]);
-            const float sc = 1.f / fmaxf(1.f, sqrtf(a1 * a1 + a2 * a2));
-            n1[o] = a1 * sc;
-            n2[o] = a2 * sc;
-        }
-        __syncthreads();
+    if (pair) return in0 ? *reinterpret_cast<const float2 *>(p + off) : make_float2(0.f, 0.f);
+    return make_float2(in0 ? p[off] : 0.f, in1 ? p[off + 1] : 0.f);
+}
+
+__device__ __forceinline__ void st_pair(float *p, int off, float2 v, bool in0, bool in1, int pair)
+{
+    if (pair) {
+        if (in0) *reinterpret_cast<float2 *>(p + off) = v;
+    } else {
+        if (in0) p[off] = v.x;
+        if (in1) p[off + 1] = v.y;
     }
 }
 
-// u_n = h - theta div p; d_n = w_n - u_n.
-__global__ void prox_out_kernel(const float *__restrict__ P, const float *__restrict__ Hb, Geo g,
-                                float theta, const float *__restrict__ Wn, float *__restrict__ Un,
-                                float *__restrict__ Dn)
-{
-    const size_t p = blockIdx.x * (size_t)kT + threadIdx.x;
-    const int bi = blockIdx.y;
-    if (p >= g.HW()) return;
-    const int i = (int)(p / g.W), j = (int)(p % g.W);
-    const float *p1 = P + (size_t)bi * 2 * g.HW(), *p2 = p1 + g.HW();
-    const float u = Hb[bi * g.HW() + p] - theta * divp(p1, p2, i, j, g.H, g.W);
-    const size_t o = bi * g.NV() + p;
-    Un[o] = u;
-    if (Dn) Dn[o] = Wn[o] - u;
-}
-
-// Reverse of prox_out: ubar -> hbar (set), pbar^T = theta grad ubar; theta
-// partial -<ubar, div p^T> into acc[2].
-__global__ void prox_out_bwd_kernel(const float *__restrict__ P, Geo g, float theta,
-                                    const float *__restrict__ Ubar_n, float *__restrict__ Hbar,
-                                    float *__restrict__ Pbar, double *__restrict__ acc)
-{
-    const size_t p = blockIdx.x * (size_t)kT + threadIdx.x;
-    const int bi = blockIdx.y;
-    double tb = 0.0;
-    if (p < g.HW()) {
-        const int i = (int)(p / g.W), j = (int)(p % g.W);
-        const float *p1 = P + (size_t)bi * 2 * g.HW(), *p2 = p1 + g.HW();
-        const float *ub = Ubar_n + (size_t)bi * g.NV();
-        const float uc = ub[p];
-        Hbar[bi * g.HW() + p] = uc;
-        tb = (double)(-uc * divp(p1, p2, i, j, g.H, g.W));
-        // d/dp of -theta <ubar, div p> = theta grad ubar (div = -grad^T)
-        float *b1 = Pbar + (size_t)bi * 2 * g.HW(), *b2 = b1 + g.HW();
-        b1[p] = i < g.H - 1 ? theta * (ub[p + g.W] - uc) : 0.f;
-        b2[p] = j < g.W - 1 ? theta * (ub[p + 1] - uc) : 0.f;
-    }
-    block_acc(tb, acc, 2);
-}
-
-// Reverse of one dual step p^{t+1} = proj(a), a = p^t + tau (grad q - kappa
-// p^t), q = div p^t - h / theta.  Given pbar^{t+1}:
-//   abar  = J_proj(a)^T pbar^{t+1}   (J = (I - a a^T / |a|^2) / |a| if |a| > 1)
-//   qbar  = tau grad^T abar = -tau div abar
-//   pbar^t = (1 - tau kappa) abar - grad qbar,  hbar -= qbar / theta,
-// and the theta partials: kappa = eps / theta gives -tau <abar, p^t> (-eps /
-// theta^2), the h / theta term gives <qbar, h> / theta^2.
-// One pass: a CTA owns a 28 x 28 tile of one batch item and keeps a 32 x 32
-// region (2 pixels of halo on every side) in shared memory, one region column
-// per lane and kRB rows per warp: q on the region, abar where qbar needs it,
-// qbar one row / column beyond the tile, then pbar^t and hbar on the tile;
-// abar never leaves the chip.  The theta partials are summed over the tile's
-// own pixels only (in FP32 per thread, FP64 from the block sum on).
-constexpr int kBT = 28;              // tile side
-constexpr int kDR = kBT + 4;         // region side: one warp's 32 lanes
-constexpr int kDP = kDR + 1;         // row pitch
-static_assert(kDR == 32, "one region column per lane");
-
-__global__ void __launch_bounds__(kT) dual_bwd_kernel(const DualArgs A,
-                                                      const float *__restrict__ Pbar_next,
-                                                      float *__restrict__ Pbar,
-                                                      float *__restrict__ Hbar, float eps,
-                                                      double *__restrict__ acc)
-{
-    // p^t, overwritten by abar where it is formed (each pixel reads only its own
-    // p there); q, then qbar
-    __shared__ float sp1[kDR][kDP], sp2[kDR][kDP], sh[kDR][kDP], sq[kDR][kDP];
-    float(&sa1)[kDR][kDP] = sp1;
-    float(&sa2)[kDR][kDP] = sp2;
-    float(&sqb)[kDR][kDP] = sq;
-    constexpr int kW = kT / 32;  // warps
-    const Geo &g = A.g;
-    const int H = g.H, W = g.W;
-    const int tx = (W + kBT - 1) / kBT;
-    const int i0 = (int)(blockIdx.x / tx) * kBT, j0 = (int)(blockIdx.x % tx) * kBT;
-    const int bi = blockIdx.y;
-    const int lj = (int)(threadIdx.x & 31), wr = (int)(threadIdx.x >> 5);
-    const int j = j0 - 2 + lj;  // the lane's image column
-    const bool cin = j >= 0 && j < W;
-    const size_t HW = g.HW();
-    const float *p1 = A.P + (size_t)bi * 2 * HW, *p2 = p1 + HW;
-    const float *h = A.Hb + (size_t)bi * HW;
-    const float *n1 = Pbar_next + (size_t)bi * 2 * HW, *n2 = n1 + HW;
-    // local (li, lj) is image (i0 - 2 + li, j0 - 2 + lj); outside the image 0
-    for (int li = wr; li < kDR; li += kW) {
-        const int i = i0 - 2 + li;
-        const bool in = cin && i >= 0 && i < H;
-        const int o = in ? i * W + j : 0;  // H W < 2^31
-        sp1[li][lj] = in ? p1[o] : 0.f;
-        sp2[li][lj] = in ? p2[o] : 0.f;
-        sh[li][lj] = in ? h[o] : 0.f;
-    }
-    __syncthreads();
-    // q = div p - h / theta on local rows / columns 1 .. 31 (boundaries as divp)
-    if (lj >= 1) {
-        for (int li = 1 + wr; li < kDR; li += kW) {
-            const int i = i0 - 2 + li;
-            const float a = (i < H - 1 ? sp1[li][lj] : 0.f) - (i > 0 ? sp1[li - 1][lj] : 0.f);
-            const float c = (j < W - 1 ? sp2[li][lj] : 0.f) - (j > 0 ? sp2[li][lj - 1] : 0.f);
-            sq[li][lj] = (a + c) - sh[li][lj] * A.inv_theta;
+// The lane's place in the region (the same for both directions).
+template <int NW, int RPW>
+struct HuberTile {
+    int lane, wp, gi0, gc, r0, j0;
+    bool in0, in1, own0, own1, interior;
+    bool mc0, mc1;           // the columns have a column to their right in the image
+    unsigned inr, ownr, mr;  // bit i: row i in the image / owned / has a row below it
+    __device__ __forceinline__ HuberTile(const HuberArgs &a)
+    {
+        constexpr int RH = NW * RPW + 2;
+        const int H = a.g.H, W = a.g.W;
+        const int bx = (int)blockIdx.x % a.tx, by = (int)blockIdx.x / a.tx;
+        lane = (int)(threadIdx.x & 31);
+        wp = (int)(threadIdx.x >> 5);
+        gi0 = by * a.TH - a.hh;
+        const int gj0 = bx * a.TW - a.hc;
+        j0 = 2 * lane;
+        gc = gj0 + j0;
+        r0 = 1 + wp * RPW;
+        in0 = gc >= 0 && gc < W;
+        in1 = gc + 1 >= 0 && gc + 1 < W;
+        own0 = in0 && j0 >= a.hc && j0 < a.hc + a.TW;
+        own1 = in1 && j0 + 1 >= a.hc && j0 + 1 < a.hc + a.TW;
+        mc0 = in0 && gc < W - 1;
+        mc1 = in1 && gc + 1 < W - 1;
+        interior = gi0 >= 0 && gi0 + RH < H && gj0 >= 0 && gj0 + 64 < W;
+        inr = ownr = mr = 0;
+#pragma unroll
+        for (int i = 0; i <= RPW; ++i) {
+            const int gi = gi0 + r0 + i;
+            if (gi >= 0 && gi < H) inr |= 1u << i;
+            if (gi >= 0 && gi < H - 1) mr |= 1u << i;
+            if (i < RPW && gi >= 0 && gi < H && r0 + i >= a.hh && r0 + i < a.hh + a.TH)
+                ownr |= 1u << i;
         }
     }
-    __syncthreads();
-    const float theta = 1.f / A.inv_theta;
-    const float kfac = -A.tau * (-eps / (theta * theta));
-    const bool ctile = lj >= 2 && lj < kBT + 2 && j < W;
-    float tk = 0.f, tq = 0.f;  // this thread's theta partials (tile pixels)
-    // abar on local rows / columns 1 .. 30
-    if (lj >= 1 && lj < kDR - 1) {
-        for (int li = 1 + wr; li < kDR - 1; li += kW) {
-            const int i = i0 - 2 + li;
-            const float qc = sq[li][lj];
-            const float gx = i < H - 1 ? sq[li + 1][lj] - qc : 0.f;
-            const float gy = j < W - 1 ? sq[li][lj + 1] - qc : 0.f;
-            const float pc1 = sp1[li][lj], pc2 = sp2[li][lj];
-            const float a1 = pc1 + A.tau * (gx - A.kappa * pc1);
-            const float a2 = pc2 + A.tau * (gy - A.kappa * pc2);
-            const bool in = cin && i >= 0 && i < H;
-            const int o = in ? i * W + j : 0;
-            const float b1 = in ? n1[o] : 0.f, b2 = in ? n2[o] : 0.f;
-            const float na = sqrtf(a1 * a1 + a2 * a2);
-            float o1 = b1, o2 = b2;
-            if (na > 1.f) {  // J = (I - a a^T / |a|^2) / |a|, symmetric
-                const float inv = 1.f / na;
-                const float dot = (a1 * b1 + a2 * b2) * inv * inv;
-                o1 = (b1 - a1 * dot) * inv;
-                o2 = (b2 - a2 * dot) * inv;
+    __device__ __forceinline__ int off(int i, int W) const { return (gi0 + r0 + i) * W + gc; }
+    __device__ __forceinline__ bool row_in(int i) const { return (inr >> i) & 1u; }
+    __device__ __forceinline__ bool row_own(int i) const { return (ownr >> i) & 1u; }
+    // zero a row component without a row below, a column component without a column to the right
+    __device__ __forceinline__ void mask(int i, float2 &x, float2 &y) const
+    {
+        if (!((mr >> i) & 1u)) x = make_float2(0.f, 0.f);
+        y.x = mc0 ? y.x : 0.f;
+        y.y = mc1 ? y.y : 0.f;
+    }
+};
+
+// Programmatic dependent launch: lets the next launch's blocks start (they wait
+// here too), then waits until the launch before has completed and its writes
+// are visible.  Every thread calls it before its first access to memory.
+__device__ __forceinline__ void pdl_enter()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
+
+// 1 / max(1, |a|) of a lane's two columns.  Square root and reciprocal by
+// Markstein's FMA residual corrections (P. Markstein, "IA-64 and Elementary
+// Functions", 2000) of the approximate reciprocal root, packed and free of
+// branches: sqrtf and the division take a slow-path branch each, which keeps a
+// warp's rows from overlapping (forward of 8 x 16 x 512 x 512, 5 iterations: 15.6
+// against 11.3 ms).  The reciprocal starts one ulp high, which settles the roots
+// with an all-ones mantissa.  For every finite |a|^2 >= 1 the result equals
+// 1.f / sqrtf(|a|^2) (all 2^30 of them compared on this GPU): the iterates stand on
+// the kink of the projection, where one ulp can flip a gradient's branch.  |a|^2
+// overflowing gives 0 and NaN gives 1, as 1.f / fmaxf(1.f, sqrtf(|a|^2)) does.
+__device__ __forceinline__ float2 huber_scale(float2 a1, float2 a2)
+{
+    const float2 s = fma2(a1, a1, mul2(a2, a2));
+    const float2 m = make_float2(fmaxf(s.x, 1.f), fmaxf(s.y, 1.f));
+    float2 y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.x) : "f"(m.x));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y.y) : "f"(m.y));
+    const float2 g = mul2(m, y), ng = mul2(m, mul2(y, splat(-1.f)));
+    const float2 r = fma2(ng, g, m);                           // m - g^2, exact
+    const float2 nroot = fma2(r, mul2(y, splat(-0.5f)), ng);   // -sqrt(m)
+    const float2 yb = fma2(y, splat(1.1920929e-7f), y);
+    const float2 e = fma2(nroot, yb, splat(1.f));
+    const float2 x = fma2(e, fma2(e, yb, yb), yb);
+    return make_float2(fmaxf(x.x, 0.f), fmaxf(x.y, 0.f));  // NaN (overflow) to 0
+}
+
+template <bool INTERIOR, int NW, int RPW>
+__device__ __forceinline__ void huber_steps(const HuberArgs &a, const HuberTile<NW, RPW> &t,
+                                            Bnd<NW> &sb, float2 (&p1)[RPW], float2 (&p2)[RPW],
+                                            const float2 (&h)[RPW + 1], float *rec)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const size_t step = (size_t)a.g.B * 2 * a.g.HW();
+    const int HW = (int)a.g.HW();
+    const int lo = a.hh - (a.Pout ? 0 : 1), hi = a.hh + a.TH;
+    for (int st = 0; st < a.ns; ++st) {
+        const int par = st & 1, nxt = par ^ 1;
+        const int e = a.ns - 1 - st;
+        if (t.r0 + RPW > lo - e && t.r0 < hi + e) {
+            const float2 pu0 = sb.up[par][t.wp][t.lane];
+            const float2 dn1 = sb.dn1[par][t.wp][t.lane], dn2 = sb.dn2[par][t.wp][t.lane];
+            float2 qc = q_pair(p1[0], pu0, p2[0], __shfl_up_sync(FULL, p2[0].y, 1), h[0],
+                               a.inv_theta);
+#pragma unroll
+            for (int i = 0; i < RPW; ++i) {
+                const float2 qn =
+                    i + 1 < RPW
+                        ? q_pair(p1[i + 1 < RPW ? i + 1 : 0], p1[i], p2[i + 1 < RPW ? i + 1 : 0],
+                                 __shfl_up_sync(FULL, p2[i + 1 < RPW ? i + 1 : 0].y, 1), h[i + 1],
+                                 a.inv_theta)
+                        : q_pair(dn1, p1[RPW - 1], dn2, __shfl_up_sync(FULL, dn2.y, 1), h[RPW],
+                                 a.inv_theta);
+                const float qr = __shfl_down_sync(FULL, qc.x, 1);
+                float2 gx = sub2(qn, qc), gy = make_float2(qc.y - qc.x, qr - qc.y);
+                if (!INTERIOR) t.mask(i, gx, gy);
+                const float2 a1 = fma2(splat(a.tau), fma2(splat(-a.kappa), p1[i], gx), p1[i]);
+                const float2 a2 = fma2(splat(a.tau), fma2(splat(-a.kappa), p2[i], gy), p2[i]);
+                if (rec && t.row_own(i)) {
+                    float *r = rec + st * step;
+                    const int o = t.off(i, a.g.W);
+                    st_pair(r, o, a1, t.own0, t.own1, a.pair);
+                    st_pair(r + HW, o, a2, t.own0, t.own1, a.pair);
+                }
+                const float2 sc = huber_scale(a1, a2);
+                p1[i] = mul2(a1, sc);
+                p2[i] = mul2(a2, sc);
+                qc = qn;
             }
-            sa1[li][lj] = o1;
-            sa2[li][lj] = o2;
-            // kappa = eps / theta: d/dtheta of -tau kappa <abar, p>
-            if (ctile && li >= 2 && li < kBT + 2 && i < H) tk += o1 * pc1 + o2 * pc2;
+            if (t.wp + 1 < NW) sb.up[nxt][t.wp + 1][t.lane] = p1[RPW - 1];
+            if (t.wp > 0) {
+                sb.dn1[nxt][t.wp - 1][t.lane] = p1[0];
+                sb.dn2[nxt][t.wp - 1][t.lane] = p2[0];
+            }
         }
+        __syncthreads();
+    }
+}
+
+template <int NW, int RPW>
+__global__ void __launch_bounds__(NW * 32, 2) huber_fwd_kernel(const HuberArgs a)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int RH = NW * RPW + 2;
+    __shared__ Bnd<NW> sb;
+    const HuberTile<NW, RPW> t(a);
+    pdl_enter();
+    const int W = a.g.W, bi = blockIdx.y, lane = t.lane, wp = t.wp;
+    const size_t HW = a.g.HW();
+    const float *Wn = a.Wn + bi * a.g.NV(), *A = a.A + bi * a.g.NV(), *C = a.C + bi * a.g.NV();
+    float *Hb = a.Hb + bi * HW;
+    float2 p1[RPW], p2[RPW], h[RPW + 1];
+    float2 f1 = make_float2(0.f, 0.f), f2 = f1;
+    if (a.Pin) {
+        const float *P1 = a.Pin + (size_t)bi * 2 * HW, *P2 = P1 + HW;
+#pragma unroll
+        for (int i = 0; i <= RPW; ++i) {
+            const bool i0 = t.row_in(i) && t.in0, i1 = t.row_in(i) && t.in1;
+            h[i] = ld_pair(Hb, t.off(i, W), i0, i1, a.pair);
+            if (i < RPW) {
+                p1[i < RPW ? i : 0] = ld_pair(P1, t.off(i, W), i0, i1, a.pair);
+                p2[i < RPW ? i : 0] = ld_pair(P2, t.off(i, W), i0, i1, a.pair);
+            }
+        }
+        if (wp == 0 || wp == NW - 1) {  // frozen rows 0 and RH - 1 of the region
+            const int gi = t.gi0 + (wp == 0 ? 0 : RH - 1);
+            if (gi >= 0 && gi < a.g.H) {
+                f1 = ld_pair(P1, gi * W + t.gc, t.in0, t.in1, a.pair);
+                f2 = ld_pair(P2, gi * W + t.gc, t.in0, t.in1, a.pair);
+            }
+        }
+    } else {
+        const float rho = a.rho, gam = a.gam, den = a.rho + 2.f * a.gam;
+#pragma unroll
+        for (int i = 0; i <= RPW; ++i) {
+            const bool i0 = t.row_in(i) && t.in0, i1 = t.row_in(i) && t.in1;
+            const int o = t.off(i, W);
+            const float2 w = ld_pair(Wn, o, i0, i1, a.pair);
+            float2 s = make_float2(0.f, 0.f);
+            if (gam > 0.f) s = add2(ld_pair(A, o, i0, i1, a.pair), ld_pair(C, o, i0, i1, a.pair));
+            // the roundings of the numerator are written out: the iterates reach the
+            // kink of the projection, where a changed bit can flip a gradient's branch
+            h[i].x = __fmaf_rn(gam, s.x, __fmul_rn(rho, w.x)) / den;
+            h[i].y = __fmaf_rn(gam, s.y, __fmul_rn(rho, w.y)) / den;
+            if (i < RPW && t.row_own(i)) st_pair(Hb, o, h[i], t.own0, t.own1, a.pair);
+        }
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) p1[i] = p2[i] = make_float2(0.f, 0.f);
+    }
+    if (wp == 0) sb.up[0][0][lane] = sb.up[1][0][lane] = f1;
+    if (wp == NW - 1) {
+        sb.dn1[0][NW - 1][lane] = sb.dn1[1][NW - 1][lane] = f1;
+        sb.dn2[0][NW - 1][lane] = sb.dn2[1][NW - 1][lane] = f2;
+    }
+    if (wp + 1 < NW) sb.up[0][wp + 1][lane] = p1[RPW - 1];
+    if (wp > 0) {
+        sb.dn1[0][wp - 1][lane] = p1[0];
+        sb.dn2[0][wp - 1][lane] = p2[0];
     }
     __syncthreads();
-    // qbar = -tau div abar on local rows / columns 2 .. 30
-    if (lj >= 2 && lj < kDR - 1) {
-        for (int li = 2 + wr; li < kDR - 1; li += kW) {
-            const int i = i0 - 2 + li;
-            const float a = (i < H - 1 ? sa1[li][lj] : 0.f) - (i > 0 ? sa1[li - 1][lj] : 0.f);
-            const float c = (j < W - 1 ? sa2[li][lj] : 0.f) - (j > 0 ? sa2[li][lj - 1] : 0.f);
-            sqb[li][lj] = -A.tau * (a + c);
+    float *rec = a.rec ? a.rec + (size_t)bi * 2 * HW : nullptr;
+    if (t.interior) huber_steps<true, NW, RPW>(a, t, sb, p1, p2, h, rec);
+    else huber_steps<false, NW, RPW>(a, t, sb, p1, p2, h, rec);
+    if (a.Pout) {
+        float *Q1 = a.Pout + (size_t)bi * 2 * HW, *Q2 = Q1 + HW;
+#pragma unroll
+        for (int i = 0; i < RPW; ++i)
+            if (t.row_own(i)) {
+                st_pair(Q1, t.off(i, W), p1[i], t.own0, t.own1, a.pair);
+                st_pair(Q2, t.off(i, W), p2[i], t.own0, t.own1, a.pair);
+            }
+    } else if (a.Un) {
+        float *Un = a.Un + bi * a.g.NV(), *Dn = a.Dn + bi * a.g.NV();
+        const float2 pu0 = sb.up[a.ns & 1][wp][lane];
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+            const float p2l = __shfl_up_sync(FULL, p2[i].y, 1);
+            const float2 dv = add2(sub2(p1[i], i == 0 ? pu0 : p1[i > 0 ? i - 1 : 0]),
+                                   sub2(p2[i], make_float2(p2l, p2[i].x)));
+            if (!t.row_own(i)) continue;
+            const int o = t.off(i, W);
+            const float2 u = fma2(splat(-a.theta), dv, h[i]);
+            st_pair(Un, o, u, t.own0, t.own1, a.pair);
+            st_pair(Dn, o, sub2(ld_pair(Wn, o, t.own0, t.own1, a.pair), u), t.own0, t.own1, a.pair);
         }
     }
-    __syncthreads();
-    // pbar^t = (1 - tau kappa) abar - grad qbar; hbar -= qbar / theta (tile)
-    const float damp = 1.f - A.tau * A.kappa;
-    float *pb1 = Pbar + (size_t)bi * 2 * HW, *pb2 = pb1 + HW;
-    float *hb = Hbar + (size_t)bi * HW;
-    if (ctile) {
-        for (int li = 2 + wr; li < kBT + 2; li += kW) {
-            const int i = i0 - 2 + li;
-            if (i >= H) break;
-            const int o = i * W + j;
-            const float qc = sqb[li][lj];
-            const float gx = i < H - 1 ? sqb[li + 1][lj] - qc : 0.f;
-            const float gy = j < W - 1 ? sqb[li][lj + 1] - qc : 0.f;
-            pb1[o] = damp * sa1[li][lj] - gx;
-            pb2[o] = damp * sa2[li][lj] - gy;
-            hb[o] -= qc * A.inv_theta;
-            tq += qc * sh[li][lj];
+}
+
+// The recorded a of the lane's rows, fetched kRing - 1 steps ahead into shared
+// memory by asynchronous copies.  Every thread reads back only what it copied
+// itself, so a wait on its own copies is all the ordering needed, and the
+// fetches cost no registers.
+constexpr int kRing = 4;
+
+template <int NW, int RPW>
+struct HuberRing {
+    static constexpr int kSlot = 2 * RPW * NW * 32;  // float2 per step
+    static constexpr size_t bytes() { return sizeof(float2) * kRing * kSlot; }
+    float2 *buf;           // the thread's column of the ring
+    const float *src[RPW];  // the row in the a of the step to fetch next
+    size_t step;           // floats between steps
+    int hw, pair;
+    unsigned in0, in1;     // bit i: the row's columns are in the image
+
+    __device__ __forceinline__ HuberRing(const HuberArgs &a, const HuberTile<NW, RPW> &t,
+                                         const float *rec, int first, float2 *mem)
+        : buf(mem + threadIdx.x), step((size_t)a.g.B * 2 * a.g.HW()), hw((int)a.g.HW()),
+          pair(a.pair), in0(t.in0 ? t.inr : 0u), in1(t.in1 ? t.inr : 0u)
+    {
+#pragma unroll
+        for (int i = 0; i < RPW; ++i)  // outside the image any valid address (nothing is read)
+            src[i] = rec + (size_t)first * step + ((in0 >> i) & 1u ? t.off(i, a.g.W) : 0);
+    }
+    // Fetches the rows of the next step (going down) as one group of copies into
+    // slot `slot`; an empty group when there is none.
+    __device__ __forceinline__ void fetch(int slot, bool any)
+    {
+        if (any) {
+            const unsigned d = (unsigned)__cvta_generic_to_shared(buf + slot * kSlot);
+#pragma unroll
+            for (int i = 0; i < RPW; ++i) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const unsigned dst = d + (unsigned)((c * RPW + i) * NW * 32 * sizeof(float2));
+                    const float *q = src[i] + (c ? hw : 0);
+                    if (pair) {
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst),
+                                     "l"(q), "r"(((in0 >> i) & 1u) * 8)
+                                     : "memory");
+                    } else {
+                        // gc is even, so a second column in the image has the first there too
+                        const unsigned x = (in0 >> i) & 1u, y = (in1 >> i) & 1u;
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst),
+                                     "l"(q), "r"(x * 4)
+                                     : "memory");
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4),
+                                     "l"(q + (x & y)), "r"(y * 4)
+                                     : "memory");
+                    }
+                }
+                src[i] -= step;
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    // all but the newest kRing - 2 groups of this thread have arrived
+    __device__ __forceinline__ void wait() const
+    {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");
+    }
+    __device__ __forceinline__ float2 get(int slot, int c, int i) const
+    {
+        return buf[slot * kSlot + (c * RPW + i) * NW * 32];
+    }
+};
+
+// Reverse of steps t0 + ns - 1 .. t0 on the region.  Needs a of t0 - 1 too (the
+// theta partial takes p^{t0}).  Step st's a is group st of the ring.
+template <bool INTERIOR, int NW, int RPW>
+__device__ __forceinline__ void huber_reverse(const HuberArgs &a, const HuberTile<NW, RPW> &t,
+                                              Bnd<NW> &sb, HuberRing<NW, RPW> &ring, int groups,
+                                              float2 (&b1)[RPW], float2 (&b2)[RPW],
+                                              float2 (&sq)[RPW], float &tk, float &tk_err)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const float damp = 1.f - a.tau * a.kappa;
+    const int lo = a.hh, hi = a.hh + a.TH;
+    float2 a1[RPW], a2[RPW], inv[RPW];  // a of the step, 1 / max(1, |a|)
+    ring.wait();
+#pragma unroll
+    for (int i = 0; i < RPW; ++i) {
+        a1[i] = ring.get(0, 0, i);
+        a2[i] = ring.get(0, 1, i);
+        inv[i] = huber_scale(a1[i], a2[i]);
+    }
+    int e = a.ns - 1;
+    for (int st = 0; st < a.ns; ++st, --e) {
+        const int par = st & 1;
+        const bool live = t.r0 + RPW > lo - e - 1 && t.r0 < hi + e + 1;
+        if (live) {
+#pragma unroll
+            for (int i = 0; i < RPW; ++i) {
+                const float2 dot =
+                    mul2(fma2(a1[i], b1[i], mul2(a2[i], b2[i])), mul2(inv[i], inv[i]));
+                const float2 nd = mul2(dot, splat(-1.f));
+                const float2 o1 = mul2(fma2(a1[i], nd, b1[i]), inv[i]);
+                const float2 o2 = mul2(fma2(a2[i], nd, b2[i]), inv[i]);
+                // |a| <= 1 (inv = 1): the projection is the identity
+                b1[i].x = inv[i].x < 1.f ? o1.x : b1[i].x;
+                b1[i].y = inv[i].y < 1.f ? o1.y : b1[i].y;
+                b2[i].x = inv[i].x < 1.f ? o2.x : b2[i].x;
+                b2[i].y = inv[i].y < 1.f ? o2.y : b2[i].y;
+                if (!INTERIOR) t.mask(i, b1[i], b2[i]);
+            }
+            if (t.wp + 1 < NW) sb.up[par][t.wp + 1][t.lane] = b1[RPW - 1];
+            if (t.wp > 0) {
+                sb.dn1[par][t.wp - 1][t.lane] = b1[0];
+                sb.dn2[par][t.wp - 1][t.lane] = b2[0];
+            }
+        }
+        __syncthreads();
+        if (live) {
+            // group st + 3 into the slot that group st - 1 has left
+            ring.fetch((st + kRing - 1) % kRing, st + kRing - 1 < groups);
+            ring.wait();  // group st + 1
+            const float2 pu0 = sb.up[par][t.wp][t.lane];
+            const float2 dn1 = sb.dn1[par][t.wp][t.lane], dn2 = sb.dn2[par][t.wp][t.lane];
+            // p^t = n / max(1, |n|), n the a of the step before: the theta partial
+            // <abar, p^t> of the own tile
+            float2 part = make_float2(0.f, 0.f);
+            const bool more = st + 1 < groups;
+#pragma unroll
+            for (int i = 0; i < RPW; ++i) {
+                a1[i] = a2[i] = make_float2(0.f, 0.f);
+                if (more) {
+                    a1[i] = ring.get((st + 1) % kRing, 0, i);
+                    a2[i] = ring.get((st + 1) % kRing, 1, i);
+                }
+                inv[i] = huber_scale(a1[i], a2[i]);
+                const float2 w = mul2(fma2(b1[i], a1[i], mul2(b2[i], a2[i])), inv[i]);
+                if (t.row_own(i)) part = add2(part, w);
+            }
+            const float p = (t.own0 ? part.x : 0.f) + (t.own1 ? part.y : 0.f);
+            const float s = tk + p, v = s - tk;  // two-sum
+            tk_err += (tk - (s - v)) + (p - v);
+            tk = s;
+            auto q_of = [&](float2 x1, float2 up, float2 x2) {
+                const float l = __shfl_up_sync(FULL, x2.y, 1);
+                return mul2(splat(-a.tau),
+                            add2(sub2(x1, up), make_float2(x2.x - l, x2.y - x2.x)));
+            };
+            float2 qc = q_of(b1[0], pu0, b2[0]);
+#pragma unroll
+            for (int i = 0; i < RPW; ++i) {
+                const float2 qn = i + 1 < RPW ? q_of(b1[i + 1 < RPW ? i + 1 : 0], b1[i],
+                                                     b2[i + 1 < RPW ? i + 1 : 0])
+                                              : q_of(dn1, b1[RPW - 1], dn2);
+                const float qr = __shfl_down_sync(FULL, qc.x, 1);
+                float2 gx = sub2(qc, qn), gy = make_float2(qc.x - qc.y, qc.y - qr);  // -grad
+                if (!INTERIOR) t.mask(i, gx, gy);
+                sq[i] = add2(sq[i], qc);
+                b1[i] = fma2(splat(damp), b1[i], gx);
+                b2[i] = fma2(splat(damp), b2[i], gy);
+                qc = qn;
+            }
         }
     }
-    block_acc((double)tk * (double)kfac + (double)tq * ((double)A.inv_theta * A.inv_theta), acc,
-              2);
+    asm volatile("cp.async.wait_all;" ::: "memory");  // of warps that stopped early
+}
+
+template <int NW, int RPW>
+__global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(const HuberArgs a)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    __shared__ Bnd<NW> sb;
+    const HuberTile<NW, RPW> t(a);
+    pdl_enter();
+    const int W = a.g.W, H = a.g.H, bi = blockIdx.y, lane = t.lane, wp = t.wp;
+    const size_t HW = a.g.HW();
+    const float *rec = a.rec + (size_t)bi * 2 * HW;
+    extern __shared__ float2 s_ring[];
+    // a of steps t0 + ns - 1 down to t0 - 1 (none before step 0)
+    const int groups = a.ns + (a.t0 > 0);
+    HuberRing<NW, RPW> ring(a, t, rec, a.t0 + a.ns - 1, s_ring);
+    for (int q = 0; q < kRing - 1; ++q) ring.fetch(q, q < groups);
+    float *Hb = a.Hb + bi * HW, *Hbar = a.Hbar + bi * HW;
+    float2 b1[RPW], b2[RPW], sq[RPW], hb[RPW];
+    Pair32 sum[3] = {};  // theta, and in the last phase rho, gamma
+    if (a.Pin) {
+        const float *P1 = a.Pin + (size_t)bi * 2 * HW, *P2 = P1 + HW;
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+            const bool i0 = t.row_in(i) && t.in0, i1 = t.row_in(i) && t.in1;
+            b1[i] = ld_pair(P1, t.off(i, W), i0, i1, a.pair);
+            b2[i] = ld_pair(P2, t.off(i, W), i0, i1, a.pair);
+        }
+    } else {
+        // pbar^T = theta grad ubar; hbar = ubar; -<ubar, div p^T>
+        const float *ub = a.Ubar + bi * a.g.NV();
+        const float *r = rec + (size_t)(a.T - 1) * a.g.B * 2 * HW;
+        auto proj = [&](int gi, float2 &x1, float2 &x2) {  // p^T of a row
+            const bool i0 = gi >= 0 && gi < H && t.in0, i1 = gi >= 0 && gi < H && t.in1;
+            x1 = ld_pair(r, gi * W + t.gc, i0, i1, a.pair);
+            x2 = ld_pair(r + HW, gi * W + t.gc, i0, i1, a.pair);
+            const float2 sc = huber_scale(x1, x2);
+            x1 = mul2(x1, sc);
+            x2 = mul2(x2, sc);
+        };
+        float2 u[RPW + 1], up1, up2;
+#pragma unroll
+        for (int i = 0; i <= RPW; ++i)
+            u[i] = ld_pair(ub, t.off(i, W), t.row_in(i) && t.in0, t.row_in(i) && t.in1, a.pair);
+        proj(t.gi0 + t.r0 - 1, up1, up2);
+        float part = 0.f;
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+            float2 x1, x2;
+            proj(t.gi0 + t.r0 + i, x1, x2);
+            const float l = __shfl_up_sync(FULL, x2.y, 1);
+            const float2 dv = add2(sub2(x1, up1), sub2(x2, make_float2(l, x2.x)));
+            up1 = x1;
+            if (t.row_own(i))
+                part -= (t.own0 ? u[i].x * dv.x : 0.f) + (t.own1 ? u[i].y * dv.y : 0.f);
+            const float ur = __shfl_down_sync(FULL, u[i].x, 1);
+            b1[i] = mul2(sub2(u[i + 1], u[i]), splat(a.theta));
+            b2[i] = mul2(sub2(make_float2(u[i].y, ur), u[i]), splat(a.theta));
+            t.mask(i, b1[i], b2[i]);
+        }
+        sum[0].hi = part;
+    }
+#pragma unroll
+    for (int i = 0; i < RPW; ++i) sq[i] = make_float2(0.f, 0.f);
+    if (wp == 0) sb.up[0][0][lane] = sb.up[1][0][lane] = make_float2(0.f, 0.f);
+    if (wp == NW - 1) {
+        sb.dn1[0][NW - 1][lane] = sb.dn1[1][NW - 1][lane] = make_float2(0.f, 0.f);
+        sb.dn2[0][NW - 1][lane] = sb.dn2[1][NW - 1][lane] = make_float2(0.f, 0.f);
+    }
+    float tk = 0.f, tk_err = 0.f;
+    if (t.interior) huber_reverse<true, NW, RPW>(a, t, sb, ring, groups, b1, b2, sq, tk, tk_err);
+    else huber_reverse<false, NW, RPW>(a, t, sb, ring, groups, b1, b2, sq, tk, tk_err);
+    // hbar -= sum qbar / theta and the h / theta partial <qbar, h> / theta^2
+    const float *ub = a.Ubar + bi * a.g.NV();
+    float tq = 0.f;
+    float2 h[RPW];
+#pragma unroll
+    for (int i = 0; i < RPW; ++i) {
+        const bool o0 = t.row_own(i) && t.own0, o1 = t.row_own(i) && t.own1;
+        const int o = t.off(i, W);
+        h[i] = ld_pair(Hb, o, o0, o1, a.pair);
+        hb[i] = ld_pair(a.Pin ? Hbar : ub, o, o0, o1, a.pair);
+        hb[i] = fma2(sq[i], splat(-a.inv_theta), hb[i]);
+        tq += (o0 ? sq[i].x * h[i].x : 0.f) + (o1 ? sq[i].y * h[i].y : 0.f);
+    }
+    // kappa = eps / theta: d/dtheta of -tau kappa <abar, p>
+    const float it2 = a.inv_theta * a.inv_theta, kfac = a.tau * a.eps * it2;
+    sum[0].add(kfac * tk, kfac * tk_err);
+    sum[0].add(it2 * tq, 0.f);
+    if (a.Pout) {
+        float *Q1 = a.Pout + (size_t)bi * 2 * HW, *Q2 = Q1 + HW;
+#pragma unroll
+        for (int i = 0; i < RPW; ++i)
+            if (t.row_own(i)) {
+                st_pair(Q1, t.off(i, W), b1[i], t.own0, t.own1, a.pair);
+                st_pair(Q2, t.off(i, W), b2[i], t.own0, t.own1, a.pair);
+                st_pair(Hbar, t.off(i, W), hb[i], t.own0, t.own1, a.pair);
+            }
+    } else {
+        // hbar -> w_n and the neighbours; direct dL/drho, dL/dgamma
+        const float *Wn = a.Wn + bi * a.g.NV(), *A = a.A + bi * a.g.NV(), *C = a.C + bi * a.g.NV();
+        float *Wb = a.Wbar + bi * a.g.NV(), *Ab = a.Abar + bi * a.g.NV(),
+              *Cb = a.Cbar + bi * a.g.NV();
+        const float den = a.rho + 2.f * a.gam, cw = a.rho / den, cn = a.gam / den;
+        float rb = 0.f, gb = 0.f;
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+            const bool o0 = t.row_own(i) && t.own0, o1 = t.row_own(i) && t.own1;
+            const int o = t.off(i, W);
+            const float2 w = ld_pair(Wn, o, o0, o1, a.pair);
+            st_pair(Wb, o, fma2(splat(cw), hb[i], ld_pair(Wb, o, o0, o1, a.pair)), o0, o1, a.pair);
+            if (a.gam > 0.f) {
+                const float2 s = add2(ld_pair(A, o, o0, o1, a.pair), ld_pair(C, o, o0, o1, a.pair));
+                st_pair(Ab, o, fma2(splat(cn), hb[i], ld_pair(Ab, o, o0, o1, a.pair)), o0, o1,
+                        a.pair);
+                st_pair(Cb, o, fma2(splat(cn), hb[i], ld_pair(Cb, o, o0, o1, a.pair)), o0, o1,
+                        a.pair);
+                gb += (o0 ? hb[i].x * (s.x - 2.f * h[i].x) / den : 0.f) +
+                      (o1 ? hb[i].y * (s.y - 2.f * h[i].y) / den : 0.f);
+            }
+            rb += (o0 ? hb[i].x * (w.x - h[i].x) / den : 0.f) +
+                  (o1 ? hb[i].y * (w.y - h[i].y) / den : 0.f);
+        }
+        sum[1].hi = rb;
+        sum[2].hi = gb;
+    }
+    if (a.Pout) {
+        Pair32 one[1] = {sum[0]};
+        const int idx[1] = {2};
+        block_acc(one, a.acc, idx);
+    } else {
+        const int idx[3] = {2, 0, 1};
+        block_acc(sum, a.acc, idx);
+    }
 }
 
 // lbar -> dL/dlogits already includes m (1 - m); Uold_bar etc. are plain adds.
@@ -430,9 +762,9 @@ struct Ws {
     float *U, *D, *Wb, *Hb, *Pa, *Pb, *PH, *Useg, *Dseg;
     float *Ubar_new, *Ubar_old, *Wbar, *Dbar, *Hbar, *Pbar_a, *Pbar_b;
     double *acc;  // [3]: rho (direct), gamma (direct), theta (total)
-    // keep_duals: the prox inputs h and dual iterates p^0..p^T of every slice of
+    // keep_duals: the prox inputs h and the a^t of the dual steps of every slice of
     // a checkpoint segment, recorded by the segment's recompute:
-    // Hall [S][Z][B][H][W], PHall [S][Z][T + 1][B][2][H][W]; else null
+    // Hall [S][Z][B][H][W], PHall [S][Z][T + 1][B][2][H][W] (T used); else null
     float *Hall, *PHall;
 };
 
@@ -488,12 +820,6 @@ struct Prm {
 };
 
 inline dim3 pgrid(const Geo &g) { return dim3((unsigned)((g.HW() + kT - 1) / kT), g.B); }
-inline dim3 grid2d(const Geo &g)
-{
-    const int rows = (g.H + kT / 32 - 1) / (kT / 32);
-    return dim3((unsigned)((g.W + 31) / 32), (unsigned)std::min(rows, 65535), g.B);
-}
-
 #define LAUNCH(kid, ...)                    \
     do {                                    \
         LaunchScope ls_((kid), s);          \
@@ -511,34 +837,170 @@ inline void neighbours(const Geo &g, int n, float *Uold, float *Unew, float *&A,
     C = n < g.Z - 1 ? Uold + (size_t)(n + 1) * HW : Unew;
 }
 
-// Runs one slice's prox (recording the dual iterates into PH when given).
-cslsm_status slice_prox(const Geo &g, const Prm &P, const float *Hb, float *Pa, float *Pb,
-                        float *PH, float **pT, cudaStream_t s)
+// Region shape (warps, rows per warp) and steps per launch.
+struct HuberShape {
+    int rpw, k;
+};
+
+inline long long huber_tiles(const Geo &g, int rpw, int k)
 {
-    const float theta = P.theta();
-    const size_t hw2 = (size_t)g.B * 2 * g.HW();
-    const int T = theta > 0.f ? P.T : 0;
-    float *cur = PH ? PH : Pa;
-    CSLSM_CUDA(cudaMemsetAsync(cur, 0, hw2 * sizeof(float), s));
-    for (int t = 0; t < T; ++t) {
-        float *nxt = PH ? PH + (size_t)(t + 1) * hw2 : (cur == Pa ? Pb : Pa);
-        DualArgs A{cur, nxt, Hb, g, 1.f / theta, P.tau, P.eps / theta};
-        LAUNCH(K_DIFF, dual_fwd_kernel<<<grid2d(g), kT, 0, s>>>(A));
-        cur = nxt;
+    const int hh = k + 1, hc = hh + (hh & 1), TH = 16 * rpw + 2 - 2 * hh, TW = 64 - 2 * hc;
+    return (long long)g.B * ((g.W + TW - 1) / TW) * ((g.H + TH - 1) / TH);
+}
+
+// Few steps and large tiles waste less work on halos, many steps need fewer
+// launches, and a launch wants a tile for every SM.  16 warps throughout (8 x 2,
+// 8 x 4 and 8 x 8 warps x rows lost at every size).  Forward + backward in ms, 5
+// iterations of 16 slices (10 for 256 x 256), steps (forward / reverse):
+//   8 x 512 x 512: 4 rows x 7 / 2 rows x 5 57.4; forward 2 rows x 7 64.6; reverse
+//     2 rows x 10 74.7, 4 rows x 10 63.6
+//   1 x 512 x 512: 2 rows x 7 / 4 rows x 7 14.2; forward 4 rows x 10 14.6, 2 rows
+//     x 10 15.7; reverse 2 rows x 10 18.0
+//   1 x 256 x 256: 2 rows x 10 / 2 rows x 7 17.4; forward 2 rows x 7 21.0, 4 rows
+//     x 10 22.0; reverse 2 rows x 10 18.2
+HuberShape huber_shape(const Geo &g, int T, bool reverse)
+{
+    HuberShape h;
+    if (reverse) {
+        if (huber_tiles(g, 2, 5) >= 600) h = {2, 5};
+        else if (huber_tiles(g, 4, 7) >= 100) h = {4, 7};
+        else h = {2, 7};
+    } else {
+        if (huber_tiles(g, 4, 7) >= 300) h = {4, 7};
+        else if (huber_tiles(g, 2, 7) >= 152) h = {2, 7};
+        else h = {2, 10};
     }
-    *pT = cur;
+    const int P = (T + h.k - 1) / h.k;  // balanced phases
+    h.k = (T + P - 1) / P;
+    return h;
+}
+
+template <int NW, int RPW>
+cslsm_status launch_huber_shape(const HuberArgs &a, dim3 grid, bool reverse, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(NW * 32);
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    LaunchScope ls(K_DIFF, s);
+    if (reverse) {
+        cfg.dynamicSmemBytes = HuberRing<NW, RPW>::bytes();
+        CSLSM_CUDA(cudaFuncSetAttribute(huber_bwd_kernel<NW, RPW>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)cfg.dynamicSmemBytes));
+        CSLSM_CUDA(cudaLaunchKernelEx(&cfg, huber_bwd_kernel<NW, RPW>, a));
+    } else {
+        CSLSM_CUDA(cudaLaunchKernelEx(&cfg, huber_fwd_kernel<NW, RPW>, a));
+    }
+    return CSLSM_OK;
+}
+
+cslsm_status launch_huber(HuberArgs a, int rpw, bool reverse, cudaStream_t s)
+{
+    a.TH = 16 * rpw + 2 - 2 * a.hh;
+    a.TW = 64 - 2 * a.hc;
+    a.tx = (a.g.W + a.TW - 1) / a.TW;
+    const dim3 grid((unsigned)(a.tx * ((a.g.H + a.TH - 1) / a.TH)), a.g.B);
+    return rpw == 2 ? launch_huber_shape<16, 2>(a, grid, reverse, s)
+                    : launch_huber_shape<16, 4>(a, grid, reverse, s);
+}
+
+inline bool pairs_ok(const Geo &g, const void *ws) { return g.W % 2 == 0 && (uintptr_t)ws % 8 == 0; }
+
+HuberArgs huber_args(const Geo &g, const Prm &P, int k, bool pair)
+{
+    HuberArgs a{};
+    a.g = g;
+    a.rho = P.rho;
+    a.gam = P.gam;
+    a.theta = P.theta();
+    a.inv_theta = 1.f / a.theta;
+    a.tau = P.tau;
+    a.eps = P.eps;
+    a.kappa = P.eps / a.theta;
+    a.T = P.T;
+    a.hh = k + 1;
+    a.hc = a.hh + (a.hh & 1);
+    a.pair = pair;
+    return a;
+}
+
+// One slice's prox of every batch item from w_n and the neighbour slices A, C:
+// h into Hb, a^t into rec [T][B][2][H][W] when given, u_n and d_n into Un, Dn
+// when given.  Pa, Pb: [B][2][H][W] scratch.
+cslsm_status slice_prox(const Geo &g, const Prm &P, const float *Wn, const float *A,
+                        const float *C, float *Hb, float *Pa, float *Pb, float *rec, float *Un,
+                        float *Dn, bool pair, cudaStream_t s)
+{
+    const HuberShape sh = huber_shape(g, P.T, false);
+    HuberArgs a = huber_args(g, P, sh.k, pair);
+    a.Wn = Wn;
+    a.A = A;
+    a.C = C;
+    a.Hb = Hb;
+    const size_t hw2 = (size_t)g.B * 2 * g.HW();
+    float *out = Pa;
+    for (int t = 0; t < P.T; t += sh.k) {
+        a.ns = std::min(sh.k, P.T - t);
+        const bool last = t + a.ns == P.T;
+        a.Pout = last ? nullptr : out;
+        a.rec = rec ? rec + (size_t)t * hw2 : nullptr;
+        a.Un = last ? Un : nullptr;
+        a.Dn = Dn;
+        cslsm_status e = launch_huber(a, sh.rpw, false, s);
+        if (e) return e;
+        a.Pin = out;
+        out = out == Pa ? Pb : Pa;
+    }
+    return CSLSM_OK;
+}
+
+// Its reverse: Ubar (dL/du_n) to Wbar, Abar, Cbar (added) and the scalars.
+cslsm_status slice_prox_bwd(const Geo &g, const Prm &P, const float *Wn, const float *A,
+                            const float *C, float *Hb, float *rec, const float *Ubar, float *Hbar,
+                            float *Pa, float *Pb, float *Wbar, float *Abar, float *Cbar,
+                            double *acc, bool pair, cudaStream_t s)
+{
+    const HuberShape sh = huber_shape(g, P.T, true);
+    HuberArgs a = huber_args(g, P, sh.k, pair);
+    a.Wn = Wn;
+    a.A = A;
+    a.C = C;
+    a.Hb = Hb;
+    a.rec = rec;
+    a.Ubar = Ubar;
+    a.Hbar = Hbar;
+    a.Wbar = Wbar;
+    a.Abar = Abar;
+    a.Cbar = Cbar;
+    a.acc = acc;
+    float *out = Pa;
+    for (int t = P.T; t > 0; t -= sh.k) {
+        a.ns = std::min(sh.k, t);
+        a.t0 = t - a.ns;
+        a.Pout = a.t0 > 0 ? out : nullptr;
+        cslsm_status e = launch_huber(a, sh.rpw, true, s);
+        if (e) return e;
+        a.Pin = out;
+        out = out == Pa ? Pb : Pa;
+    }
     return CSLSM_OK;
 }
 
 // One forward iteration on (U, D) in place; writes v when vout != null.  With
 // Hrec / PHrec (keep_duals), slice n's prox input goes to Hrec + n [B][H][W]
-// and its dual iterates to PHrec + n [T + 1][B][2][H][W].
+// and the a of its dual steps to PHrec + n [T + 1][B][2][H][W].
 cslsm_status fwd_iter(const Geo &g, const Prm &P, const float *logits, const float *b, Ws &w,
-                      float *vout, cudaStream_t s, float *Hrec = nullptr, float *PHrec = nullptr)
+                      float *vout, bool pair, cudaStream_t s, float *Hrec = nullptr,
+                      float *PHrec = nullptr)
 {
     const float gam = g.Z > 1 ? P.gam : 0.f;
     LAUNCH(K_DIFF, ux_fwd_kernel<<<pgrid(g), kT, 0, s>>>(w.U, w.D, logits, b, g, P.rho, w.Wb, vout));
-    const float theta = P.lam / (P.rho + 2.f * gam);
     Prm Q = P;
     Q.gam = gam;
     for (int n = 0; n < g.Z; ++n) {
@@ -548,12 +1010,9 @@ cslsm_status fwd_iter(const Geo &g, const Prm &P, const float *logits, const flo
         const size_t hwf = (size_t)g.B * g.HW();
         float *Hb = Hrec ? Hrec + (size_t)n * hwf : w.Hb;
         float *PH = PHrec ? PHrec + (size_t)n * (P.T + 1) * 2 * hwf : nullptr;
-        LAUNCH(K_DIFF, hform_kernel<<<pgrid(g), kT, 0, s>>>(w.Wb + off, A, C, g, P.rho, gam, Hb));
-        float *pT = nullptr;
-        cslsm_status e = slice_prox(g, Q, Hb, w.Pa, w.Pb, PH, &pT, s);
+        cslsm_status e = slice_prox(g, Q, w.Wb + off, A, C, Hb, w.Pa, w.Pb, PH, w.U + off,
+                                    w.D + off, pair, s);
         if (e) return e;
-        LAUNCH(K_DIFF, prox_out_kernel<<<pgrid(g), kT, 0, s>>>(pT, Hb, g, theta, w.Wb + off,
-                                                                 w.U + off, w.D + off));
     }
     return CSLSM_OK;
 }
@@ -581,7 +1040,8 @@ cslsm_status unrolled_forward(int B, int Z, int H, int W, float rho, float lam, 
             CSLSM_CUDA(cudaMemcpyAsync(c, w.U, nv * 4, cudaMemcpyDeviceToDevice, s));
             CSLSM_CUDA(cudaMemcpyAsync(c + nv, w.D, nv * 4, cudaMemcpyDeviceToDevice, s));
         }
-        cslsm_status e = fwd_iter(g, P, logits, b, w, k == K - 1 ? vout : nullptr, s);
+        cslsm_status e = fwd_iter(g, P, logits, b, w, k == K - 1 ? vout : nullptr,
+                                  pairs_ok(g, ws), s);
         if (e) return e;
     }
     return CSLSM_OK;
@@ -600,7 +1060,8 @@ cslsm_status unrolled_backward(int B, int Z, int H, int W, float rho, float lam,
     Ws w = carve(ws, g, T, S, keep);
     const size_t nv = (size_t)B * g.NV(), HW = g.HW(), hw2 = (size_t)B * 2 * HW;
     const size_t hwf = (size_t)B * HW;
-    const float den = rho + 2.f * gz, theta = lam / den;
+    const float den = rho + 2.f * gz;
+    const bool pair = pairs_ok(g, ws);
     CSLSM_CUDA(cudaMemsetAsync(w.acc, 0, 3 * kAccCopies * sizeof(double), s));
     CSLSM_CUDA(cudaMemsetAsync(logits_bar, 0, nv * 4, s));
     // adjoint of the state after the last iteration: only v^K is observed
@@ -622,7 +1083,7 @@ cslsm_status unrolled_backward(int B, int Z, int H, int W, float rho, float lam,
             if (k < k1) {
                 // keep_duals: record every slice's h and dual iterates of iteration k
                 cslsm_status e =
-                    fwd_iter(g, P, logits, b, w, nullptr, s,
+                    fwd_iter(g, P, logits, b, w, nullptr, pair, s,
                              keep ? w.Hall + (size_t)slot * Z * hwf : nullptr,
                              keep ? w.PHall + (size_t)slot * Z * (T + 1) * hw2 : nullptr);
                 if (e) return e;
@@ -646,34 +1107,21 @@ cslsm_status unrolled_backward(int B, int Z, int H, int W, float rho, float lam,
                 float *Ab, *Cb;
                 neighbours(g, n, w.Ubar_old, w.Ubar_new, Ab, Cb);
                 const size_t off = (size_t)n * HW;
-                const int Tn = theta > 0.f ? T : 0;
-                // the prox input h and its dual iterates p^0 .. p^T: kept by the
-                // segment's recompute, or recomputed here
-                float *Hn = w.Hb, *PHn = w.PH, *pT = nullptr;
+                // the prox input h and the a^t of its dual steps: kept by the segment's
+                // recompute, or recomputed here
+                float *Hn = w.Hb, *PHn = w.PH;
                 if (keep) {
                     Hn = w.Hall + ((size_t)slot * Z + n) * hwf;
                     PHn = w.PHall + ((size_t)slot * Z + n) * (T + 1) * hw2;
-                    pT = PHn + (size_t)Tn * hw2;
                 } else {
-                    LAUNCH(K_DIFF, hform_kernel<<<pgrid(g), kT, 0, s>>>(w.Wb + off, A, C, g, rho,
-                                                                        gz, w.Hb));
-                    cslsm_status e = slice_prox(g, P, w.Hb, w.Pa, w.Pb, w.PH, &pT, s);
+                    cslsm_status e = slice_prox(g, P, w.Wb + off, A, C, Hn, w.Pa, w.Pb, PHn,
+                                                nullptr, nullptr, pair, s);
                     if (e) return e;
                 }
-                LAUNCH(K_DIFF, prox_out_bwd_kernel<<<pgrid(g), kT, 0, s>>>(
-                                   pT, g, theta, w.Ubar_new + off, w.Hbar, w.Pbar_a, w.acc));
-                float *pb_in = w.Pbar_a, *pb_out = w.Pbar_b;
-                const dim3 tgrid((unsigned)(((W + kBT - 1) / kBT) * ((H + kBT - 1) / kBT)), B);
-                for (int t = Tn - 1; t >= 0; --t) {
-                    DualArgs Ad{PHn + (size_t)t * hw2, nullptr, Hn, g, 1.f / theta, tau,
-                                eps / theta};
-                    LAUNCH(K_DIFF, dual_bwd_kernel<<<tgrid, kT, 0, s>>>(Ad, pb_in, pb_out, w.Hbar,
-                                                                         eps, w.acc));
-                    std::swap(pb_in, pb_out);
-                }
-                LAUNCH(K_DIFF, hform_bwd_kernel<<<pgrid(g), kT, 0, s>>>(
-                                   w.Hbar, w.Wb + off, A, C, g, rho, gz, w.Wbar + off, Ab, Cb,
-                                   w.acc));
+                cslsm_status e = slice_prox_bwd(g, P, w.Wb + off, A, C, Hn, PHn,
+                                                w.Ubar_new + off, w.Hbar, w.Pbar_a, w.Pbar_b,
+                                                w.Wbar + off, Ab, Cb, w.acc, pair, s);
+                if (e) return e;
             }
             // x-update reverse: u^k, d^k adjoints
             LAUNCH(K_DIFF, ux_bwd_kernel<<<pgrid(g), kT, 0, s>>>(

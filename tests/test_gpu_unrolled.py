@@ -60,6 +60,29 @@ def test_forward_and_gradient_match_fp64_oracle(cs, B, Z, H, W):
         assert abs(ga - ge) <= 1e-3 * max(abs(ge), 1e-3), (ga, ge)
 
 
+# one pixel past a tile, odd widths (no paired accesses), one to several phases of dual
+# steps, and sizes past each line of the choice of tile and steps per launch
+@pytest.mark.parametrize("B,Z,H,W,T", [(1, 1, 1, 5, 3), (1, 2, 13, 41, 1), (2, 2, 19, 49, 7),
+                                       (1, 3, 23, 53, 11), (1, 1, 67, 96, 21),
+                                       (3, 1, 300, 301, 8), (1, 1, 520, 486, 9),
+                                       (2, 1, 620, 640, 8)])
+def test_tiled_dual_steps_match_fp64_oracle(cs, B, Z, H, W, T):
+    logits, b, _ = _problem(B + Z + H + T, B, Z, H, W)
+    vbar = torch.randn(B, Z, H, W, generator=torch.Generator().manual_seed(14))
+    cfg = dict(CFG, iters=2, tv_steps=T)
+    lg = logits.cuda().requires_grad_(True)
+    r, l_, gm = _scalars()
+    v = cs.unrolled_admm(lg, b.cuda(), r, l_, gm, **cfg)
+    (v * vbar.cuda()).sum().backward()
+    lg64 = logits.double().requires_grad_(True)
+    r64, l64, g64 = _scalars(dev="cpu", dtype=torch.float64)
+    v64 = un.unrolled_admm(lg64, b.double(), r64, l64, g64, iters=2, T=T, tau=CFG["tv_tau"],
+                           eps=CFG["huber_eps"])
+    (v64 * vbar.double()).sum().backward()
+    assert rel_l2(v.detach().cpu().numpy(), v64.detach().numpy()) <= 1e-5
+    assert rel_l2(lg.grad.cpu().numpy(), lg64.grad.numpy()) <= 1e-3
+
+
 def test_checkpoint_period_does_not_change_gradients(cs):
     logits, b, _ = _problem(5, 1, 4, 20, 18)
     vbar = torch.randn(1, 4, 20, 18, generator=torch.Generator().manual_seed(6)).cuda()
