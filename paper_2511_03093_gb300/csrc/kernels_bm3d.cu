@@ -11,19 +11,9 @@
 // on the integer SSD of the 8-bit codes clamp(rint(x*255), 0, 255).
 //
 // GB300 design.
-//  - Matching (integer ALU bound): one warp per reference.  The window's codes
-//    are staged in shared memory; lane = candidate column, and each lane walks
-//    the image rows once, keeping the partial sums of the 8 candidates that
-//    overlap the current row in a rotating register window.  The SSD is
-//    sum a^2 + sum b^2 - 2 sum ab with the cross terms from __dp4a on packed
-//    bytes (exact int32).  Each lane keeps a sorted top-15 list of 32-bit keys
-//    (SSD << 12 | window index, which orders like the global linear index);
-//    the warp merges the 32 lists with __reduce_min_sync.  Bit-exact.
-//  - Filtering (FP32): one warp per group.  Lane (k, h) holds rows 4h..4h+3 of
-//    patch k; the row DCT runs in registers, then the lane pair swaps 4x4
-//    blocks (shuffles) so that each lane holds 4 whole columns for the column
-//    DCT, and the Haar transform is a butterfly across lanes; every DCT
-//    coefficient is a compile-time constant-bank operand.
+//  - Matching: the inner products of 4 x 4 references with their joint window by
+//    mma.sync, the selection on integer keys (see the matching section).  Bit-exact.
+//  - Filtering on the tensor cores, one warp per group (see its section).
 //    A CTA owns an 8x8 block of references: it stages g (and the basic
 //    estimate) of the block's footprint in shared memory and aggregates the
 //    block's estimates there with shared atomics before one global atomic
@@ -34,6 +24,7 @@
 
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "internal.cuh"
@@ -48,9 +39,6 @@ constexpr int kStep = 3;        // reference step
 constexpr int kMaxGroup = 16;
 constexpr float kLambda3D = 2.7f;
 constexpr int kTauHard = 2500, kTauWiener = 400;
-constexpr int kWinPx = 2 * kHalfWin + kPS;  // 46 pixel rows / columns of a window
-constexpr int kWinWords = 12;               // 48 bytes per staged row
-constexpr int kMatchWarps = 8;
 constexpr int kRefBlock = 8;                // references per CTA side in the filter
 constexpr int kFoot = (kRefBlock - 1) * kStep + 2 * kHalfWin + kPS;  // 67
 constexpr int kFootPitch = kFoot + 1;
@@ -88,135 +76,478 @@ __global__ void bm3d_prep_kernel(const S *__restrict__ src, const S *__restrict_
 }
 
 // ---- block matching --------------------------------------------------------
-__device__ __forceinline__ void row_bytes(const uint32_t *row, int c, uint32_t &lo, uint32_t &hi)
+// SSD(ref, cand) = sum ref^2 + sum cand^2 - 2 <ref, cand>, and the inner products
+// of a block of references with all patches of their joint window are a matrix
+// product: one warp takes 4 x 4 references (M = 16) against the 48 x 48 candidates
+// of their windows (N, 8 adjacent columns a tile) over the 64 pixels (K), by
+// mma.sync m16n8k16 on the codes as FP16.  A = -2 ref and the accumulators start at
+// sum ref^2 + sum cand^2 + 2^23, so the product leaves SSD + 2^23; every number is
+// an integer below 2^24, so the FP32 sums are exact and the low mantissa bits of
+// the result are the SSD.
+//   B fragments: register r of a lane holds two pixels of image row r (column
+// pairs starting on odd columns come from a copy shifted by one pixel), so a tile
+// one row further down takes seven registers over and loads one.
+//   Selection: the 15 smallest (SSD, position) by 31-bit keys (SSD << 13 | window
+// row << 7 | window column, ordered like y W + x).  Pass 1 goes over the window's 16
+// middle rows; each of the 8 lanes of a reference keeps the 6 least of its pairs of
+// adjacent candidates, and the 16th smallest of those 48 SSDs bounds the 16th
+// smallest of the window (the reference itself is one).  Pass 2 forms the products
+// of the whole window and keeps the keys up to the bound (about 40), in lists of its
+// own per lane and reference; a list that fills up drops all but its 16 smallest and
+// lowers its bound.  The lanes of a reference then sort and merge their lists.
+//   Two warps share a block of references, each with every other tile column, so
+// that one small slice still gives every SM work.
+//   Measured, 4 slices of 512 x 512 (115,600 references): hard 0.683 -> 0.272 ms,
+// Wiener 0.659 -> 0.287 ms against one warp per reference on dp4a with sorted
+// insertion; 1,470 warp instructions a reference (5,530), bound by issue (57 %, integer
+// pipe 42 %, tensor pipe 29 %).  One 253 x 317 slice: 36 us of which 11 in the products
+// of pass 2.
+// mma.sync rather than tcgen05: every product goes through the ALU in the registers
+// where mma.sync leaves it, and the tensor pipe is not the limit.
+constexpr int kMSpan = 48;        // candidate rows / columns of a warp's 4 x 4 references
+constexpr int kMSide = 2;         // blocks of 4 x 4 references per CTA side
+constexpr int kMWarps = 2 * kMSide * kMSide;
+constexpr int kMCand = 3 * (4 * kMSide - 1) + 2 * kHalfWin + 1;  // 60 candidate rows / columns
+constexpr int kMPix = kMCand + kPS - 1;                          // 67 pixel rows / columns
+constexpr int kMCopy = 40;        // words per row of one copy (bank offset 8 between the two)
+constexpr int kMPitch = 2 * kMCopy;
+constexpr int kMCap = 32;         // keys per lane's list
+constexpr int kMFull = kMCap - 8; // shrunk beyond this: the next four rows bring up to 8
+constexpr int kMList = 2 * kMCap * 32;  // words per warp
+constexpr int kMFirst = 15;       // pass 1: rows 15 .. 30, in every inner reference's window
+constexpr int kMBest = 6;         // least SSDs a lane keeps in pass 1
+constexpr float kMBias = 8388608.f;  // 2^23
+constexpr float kMFar = 33554432.f;  // above every SSD + 2^23
+constexpr uint32_t kMNone = 0xffffffffu;
+constexpr size_t kMSmem = sizeof(uint32_t) * kMPix * kMPitch + sizeof(float) * kMCand * kMCand +
+                          sizeof(uint32_t) * kMWarps * (kMList + 2 * 32);
+static_assert(kMPix <= 2 * kMCopy, "a copy's row is too short");
+static_assert(kMWarps * kMList >= kMPix * kMCand, "row sums do not fit the lists' place");
+static_assert(kMCand <= 64, "13-bit window position");
+
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                         uint32_t a3, uint32_t b0, uint32_t b1)
 {
-    const int w = c >> 2, sh = (c & 3) * 8;
-    const uint32_t a = row[w], b = row[w + 1], d = row[w + 2];
-    lo = __funnelshift_r(a, b, sh);
-    hi = __funnelshift_r(b, d, sh);
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+        "{%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ void insert_key(uint32_t (&keys)[kMaxGroup - 1], uint32_t key)
+__device__ __forceinline__ void order(uint32_t &a, uint32_t &b)
 {
-    if (key >= keys[kMaxGroup - 2]) return;
+    const uint32_t lo = min(a, b);
+    b = max(a, b);
+    a = lo;
+}
+
+// Sorts 16 keys held by one lane (bitonic network).
+__device__ __forceinline__ void sort16(uint32_t (&k)[16])
+{
 #pragma unroll
-    for (int t = 0; t < kMaxGroup - 1; ++t) {
-        const uint32_t lo = min(keys[t], key);
-        key = max(keys[t], key);
-        keys[t] = lo;
+    for (int size = 2; size <= 16; size *= 2)
+#pragma unroll
+        for (int d = size / 2; d > 0; d /= 2)
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if ((i & d) == 0) {
+                    if (i & size) order(k[i | d], k[i]);
+                    else order(k[i], k[i | d]);
+                }
+}
+
+// The 16 smallest of the lane's sorted keys and 16 more (sorted, from `other`), sorted.
+template <typename F>
+__device__ __forceinline__ void merge16(uint32_t (&k)[16], F other)
+{
+    uint32_t q[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) q[i] = min(k[i], other(15 - i));
+#pragma unroll
+    for (int d = 8; d > 0; d /= 2)  // bitonic: one merge sorts them
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if ((i & d) == 0) order(q[i], q[i | d]);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) k[i] = q[i];
+}
+
+// A lane's full list down to its 16 smallest keys; returns the largest of them.
+__device__ __noinline__ uint32_t shrink_list(uint32_t *list, int n)
+{
+    uint32_t k[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) k[i] = kMNone;
+    for (int j = 0; j < n; ++j) {
+        uint32_t key = list[j * 32];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) order(k[i], key);
     }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) list[i * 32] = k[i];
+    return k[15];
 }
 
-// Walks candidate rows [ra, rb] of window column cc (local coordinates) and
-// inserts every passing candidate into the lane's list.
-__device__ __forceinline__ void scan_column(const uint32_t (*win)[kWinWords], int cc, int ra,
-                                            int rb, const uint32_t (&rlo)[kPS],
-                                            const uint32_t (&rhi)[kPS], int refsq, int thr,
-                                            int skip_l, uint32_t (&keys)[kMaxGroup - 1])
+// What a warp's lanes know about their two references (rows g and g + 8 of A) and
+// the window; columns of the references agree, rows are ylo[r] .. yhi[r] of it.
+struct MatchLane {
+    uint32_t a[4][4];  // A fragments, -2 ref
+    float base[2];     // sum ref^2 + 2^23
+    int ylo[2], yhi[2], xlo, xhi;
+    int all_lo, all_hi;  // rows valid for every reference of the warp
+    int lx, ly, t;
+};
+
+// Appends the key to the list at shared address `at` where d <= bound.  (No memory
+// clobber, so that the loads of later rows may pass it; the lists are read only in
+// a function that is not inlined or behind a warp barrier.)
+__device__ __forceinline__ void append_if(uint32_t &at, uint32_t key, float d, float bound)
 {
-    uint32_t ab[kPS];
-    uint32_t sq[kPS];
-    uint32_t sqsum = 0;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %2, %3;\n\t"
+                 "@p st.shared.u32 [%0], %1;\n\t@p add.u32 %0, %0, 128;\n\t}"
+                 : "+r"(at)
+                 : "r"(key), "f"(d), "f"(bound));
+}
+
+// What four rows of a tile column need from shared memory.
+struct MatchFetch {
+    uint32_t w[4];
+    float2 s[4];
+    __device__ __forceinline__ void load(const uint32_t *bp, const float *sp)
+    {
 #pragma unroll
-    for (int t = 0; t < kPS; ++t) ab[t] = sq[t] = 0;
-    for (int yb = ra; yb <= rb + kPS - 1; yb += kPS) {
+        for (int i = 0; i < 4; ++i) {
+            w[i] = bp[i * kMPitch];
+            s[i] = *reinterpret_cast<const float2 *>(sp + i * kMCand);
+        }
+    }
+};
+
+// Four rows (from window row y) of a tile column; R holds the pixel rows y .. y + 6,
+// and y + 4 .. y + 10 on return, f what the rows need and on return what the next
+// four need (from bp, sp).  The rows' products are four independent chains.  PASS 1:
+// SSD + 2^23 into the sorted lists best; PASS 2: keys up to the bounds vt to the
+// lists at.  WHOLE: all rows valid.
+template <int PASS, bool WHOLE>
+__device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *bp, const float *sp,
+                                           MatchFetch &f, const float (&r0)[2],
+                                           const float (&r1)[2], int y, uint32_t l,
+                                           uint32_t (&R)[7], float (&best)[2][kMBest],
+                                           uint32_t *list, uint32_t (&at)[2], float (&vt)[2])
+{
+    uint32_t w[11];
+    float d[4][4];
 #pragma unroll
-        for (int m = 0; m < kPS; ++m) {
-            const int y = yb + m;
-            if (y > rb + kPS - 1) break;
-            uint32_t lo, hi;
-            row_bytes(win[y], cc, lo, hi);
-            const uint32_t s2 = __dp4a(hi, hi, __dp4a(lo, lo, 0u));
-            sqsum += s2 - sq[m];  // running sum of b^2 over the last 8 rows
-            sq[m] = s2;
-            ab[m] = 0;  // candidate starting at row y
+    for (int i = 0; i < 7; ++i) w[i] = R[i];
 #pragma unroll
-            for (int a = 0; a < kPS; ++a) {
-                const int k = (m - a + kPS) % kPS;  // candidate row y - a
-                ab[k] = __dp4a(hi, rhi[a], __dp4a(lo, rlo[a], ab[k]));
+    for (int i = 0; i < 4; ++i) {
+        w[7 + i] = f.w[i];
+        d[i][0] = f.s[i].x + r0[0];
+        d[i][1] = f.s[i].y + r0[1];
+        d[i][2] = f.s[i].x + r1[0];
+        d[i][3] = f.s[i].y + r1[1];
+    }
+    f.load(bp, sp);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            mma16816(d[i], m.a[k][0], m.a[k][1], m.a[k][2], m.a[k][3], w[i + 2 * k],
+                     w[i + 2 * k + 1]);
+#pragma unroll
+    for (int i = 0; i < 7; ++i) R[i] = w[i + 4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool v0 = WHOLE || (unsigned)(y + i - m.ylo[0]) <= (unsigned)(m.yhi[0] - m.ylo[0]);
+        const bool v1 = WHOLE || (unsigned)(y + i - m.ylo[1]) <= (unsigned)(m.yhi[1] - m.ylo[1]);
+        if (PASS == 1) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                float v = fminf(d[i][2 * r], d[i][2 * r + 1]);
+                if (!(r ? v1 : v0)) v = kMFar;
+#pragma unroll
+                for (int j = kMBest - 1; j > 0; --j)
+                    best[r][j] = fminf(best[r][j], fmaxf(best[r][j - 1], v));
+                best[r][0] = fminf(best[r][0], v);
             }
-            const int ci = y - (kPS - 1);  // candidate finished at this row
-            if (ci >= ra) {
-                const int k = (m + 1) % kPS;
-                const int ssd = refsq + (int)sqsum - 2 * (int)ab[k];
-                const int l = ci * 64 + cc;
-                if (ssd <= thr && l != skip_l) insert_key(keys, ((uint32_t)ssd << 12) | (uint32_t)l);
+        } else {
+            const float b0 = v0 ? vt[0] : 0.f, b1 = v1 ? vt[1] : 0.f;
+            const uint32_t li = l + (uint32_t)(i * 128);
+            append_if(at[0], (__float_as_uint(d[i][0]) << 13) + li, d[i][0], b0);
+            append_if(at[1], (__float_as_uint(d[i][2]) << 13) + li, d[i][2], b1);
+            append_if(at[0], (__float_as_uint(d[i][1]) << 13) + li + 1, d[i][1], b0);
+            append_if(at[1], (__float_as_uint(d[i][3]) << 13) + li + 1, d[i][3], b1);
+        }
+    }
+    if (PASS == 2) {  // at most 8 keys more until the next look
+        const uint32_t l0 = (uint32_t)__cvta_generic_to_shared(list);
+        const uint32_t l1 = l0 + kMCap * 128;
+        if (__any_sync(0xffffffffu, at[0] > l0 + kMFull * 128 || at[1] > l1 + kMFull * 128)) {
+            if (at[0] > l0 + kMFull * 128) {
+                const uint32_t top = shrink_list(list, (int)(at[0] - l0) / 128);
+                at[0] = l0 + 16 * 128;
+                vt[0] = fminf(vt[0], kMBias + (float)(top >> 13));
             }
+            if (at[1] > l1 + kMFull * 128) {
+                const uint32_t top = shrink_list(list + kMCap * 32, (int)(at[1] - l1) / 128);
+                at[1] = l1 + 16 * 128;
+                vt[1] = fminf(vt[1], kMBias + (float)(top >> 13));
+            }
+            __syncwarp();
         }
     }
 }
 
-__global__ void __launch_bounds__(kMatchWarps * 32)
-bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int ns, int thr,
+// Walks the warp's tile columns c0, c0 + 2, c0 + 4 over rows first .. last (fours).
+template <int PASS>
+__device__ __forceinline__ void match_scan(const MatchLane &m, int c0, int first, int last,
+                                           const uint32_t *bw, const float *s_sq,
+                                           float (&best)[2][kMBest], uint32_t *list,
+                                           uint32_t (&at)[2], float (&vt)[2])
+{
+    constexpr float kPen = 16777216.f;
+    for (int c = c0; c < kMSpan / 8; c += 2) {
+        const int x = m.lx + 8 * c + 2 * m.t;
+        const bool v0 = x >= m.xlo && x <= m.xhi, v1 = x + 1 >= m.xlo && x + 1 <= m.xhi;
+        // columns outside the window: pushed above every bound
+        const float r0[2] = {m.base[0] + (v0 ? 0.f : kPen), m.base[0] + (v1 ? 0.f : kPen)};
+        const float r1[2] = {m.base[1] + (v0 ? 0.f : kPen), m.base[1] + (v1 ? 0.f : kPen)};
+        const bool any = __any_sync(0xffffffffu, v0 || v1);
+        const uint32_t *bp = bw + 4 * c + first * kMPitch;
+        const float *sp = s_sq + (m.ly + first) * kMCand + x;
+        uint32_t l = (uint32_t)((m.ly + first) * 128 + x);
+        uint32_t R[7];
+        if (!any) continue;
+#pragma unroll
+        for (int i = 0; i < 7; ++i) R[i] = bp[i * kMPitch];
+        bp += 7 * kMPitch;
+        MatchFetch f;
+        f.load(bp, sp);
+        for (int y = first; y <= last; y += 4) {
+            if (y + 4 <= last) {  // the last four rows fetch themselves again
+                bp += 4 * kMPitch;
+                sp += 4 * kMCand;
+            }
+            if (y >= m.all_lo && y + 3 <= m.all_hi)
+                match_rows<PASS, true>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
+            else
+                match_rows<PASS, false>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
+            l += 4 * 128;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kMWarps * 32, 2)
+bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
                   int *__restrict__ lists, int *__restrict__ counts, const int *__restrict__ stop)
 {
     if (stop && *stop) return;
-    __shared__ uint32_t s_win[kMatchWarps][kWinPx][kWinWords];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    uint32_t (*win)[kWinWords] = s_win[wid];
+    constexpr int kThreads = kMWarps * 32;
+    constexpr unsigned FULL = 0xffffffffu;
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint32_t *s_px = reinterpret_cast<uint32_t *>(smem);  // [kMPix][2 copies][kMCopy] FP16 pairs
+    float *s_sq = reinterpret_cast<float *>(s_px + kMPix * kMPitch);  // [kMCand][kMCand]
+    uint32_t *s_list = reinterpret_cast<uint32_t *>(s_sq + kMCand * kMCand);
+    uint32_t *s_cnt = s_list + kMWarps * kMList;  // [warp][reference g / g + 8][lane]
     const int nri = n_refs(H), nrj = n_refs(W);
-    const long long total = (long long)ns * nri * nrj;
-    for (long long t = (long long)blockIdx.x * kMatchWarps + wid; t < total;
-         t += (long long)gridDim.x * kMatchWarps) {
-        const int sl = (int)(t / ((long long)nri * nrj));
-        const int r = (int)(t - (long long)sl * nri * nrj);
-        const int ri = ref_pos(r / nrj, H), rj = ref_pos(r % nrj, W);
-        const int ci0 = max(0, ri - kHalfWin), ci1 = min(H - kPS, ri + kHalfWin);
-        const int cj0 = max(0, rj - kHalfWin), cj1 = min(W - kPS, rj + kHalfWin);
-        const int nrow = ci1 - ci0 + kPS, ncol = cj1 - cj0 + kPS;
-        const uint8_t *img = codes + (size_t)sl * H * W;
-        __syncwarp();
-        for (int idx = lane; idx < nrow * kWinWords; idx += 32) {
-            const int y = idx / kWinWords, wd = idx - y * kWinWords;
-            uint32_t v = 0;
+    constexpr int kRefs = 4 * kMSide;
+    const int tx = (nrj + kRefs - 1) / kRefs, ty = (nri + kRefs - 1) / kRefs;
+    const int sl = (int)(blockIdx.x / (unsigned)(tx * ty));
+    const int tile = (int)(blockIdx.x - (unsigned)sl * (unsigned)(tx * ty));
+    const int bi = (tile / tx) * kRefs, bj = (tile % tx) * kRefs;
+    const int oy = ref_pos(bi, H) - kHalfWin, ox = ref_pos(bj, W) - kHalfWin;
+    const uint8_t *img = codes + (size_t)sl * H * W;
+    // pixels of the joint window as FP16, pairs on even and on odd columns
+    __half *px = reinterpret_cast<__half *>(s_px);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int kChunks = (kMPix + 1 + 31) / 32;  // the last column of a copy's row is a zero
+#pragma unroll 3
+    for (int y = wid; y < kMPix; y += kMWarps) {
+        const int gy = oy + y;
+        const bool iny = gy >= 0 && gy < H;
+        int v[kChunks];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int c = wd * 4 + b;
-                if (c < ncol) v |= (uint32_t)img[(size_t)(ci0 + y) * W + cj0 + c] << (8 * b);
-            }
-            win[y][wd] = v;
+        for (int q = 0; q < kChunks; ++q) {
+            const int x = lane + 32 * q, gx = ox + x;
+            v[q] = iny && x < kMPix && gx >= 0 && gx < W ? img[(size_t)gy * W + gx] : 0;
         }
-        __syncwarp();
-        uint32_t rlo[kPS], rhi[kPS];
-        int refsq = 0;
 #pragma unroll
-        for (int a = 0; a < kPS; ++a) {
-            row_bytes(win[ri - ci0 + a], rj - cj0, rlo[a], rhi[a]);
-            refsq += (int)__dp4a(rhi[a], rhi[a], __dp4a(rlo[a], rlo[a], 0u));
-        }
-        uint32_t keys[kMaxGroup - 1];
-#pragma unroll
-        for (int k = 0; k < kMaxGroup - 1; ++k) keys[k] = 0xffffffffu;
-        const int ncc = cj1 - cj0 + 1, ncr = ci1 - ci0 + 1;  // candidate columns / rows
-        const int skip_l = (ri - ci0) * 64 + (rj - cj0);
-        if (lane < ncc) scan_column(win, lane, 0, ncr - 1, rlo, rhi, refsq, thr, skip_l, keys);
-        // columns 32..38: 7 columns x 4 row segments of 10 candidate rows
-        if (ncc > 32 && lane < 28) {
-            const int cc = 32 + lane % 7, seg = lane / 7;
-            const int ra = seg * 10, rb = min(ra + 9, ncr - 1);
-            if (cc < ncc && ra <= rb) scan_column(win, cc, ra, rb, rlo, rhi, refsq, thr, skip_l, keys);
-        }
-        int *out = lists + (size_t)t * kMaxGroup;
-        int m = 1;
-        if (lane == 0) out[0] = ri * W + rj;
-        for (; m < kMaxGroup; ++m) {
-            const uint32_t best = __reduce_min_sync(0xffffffffu, keys[0]);
-            if (best == 0xffffffffu) break;
-            if (keys[0] == best) {
-#pragma unroll
-                for (int k = 0; k < kMaxGroup - 2; ++k) keys[k] = keys[k + 1];
-                keys[kMaxGroup - 2] = 0xffffffffu;
-            }
-            if (lane == 0) {
-                const int l = (int)(best & 0xfffu);
-                out[m] = (ci0 + l / 64) * W + cj0 + l % 64;
-            }
-        }
-        if (lane == 0) {
-            for (int k = m; k < kMaxGroup; ++k) out[k] = -1;
-            counts[t] = m;
+        for (int q = 0; q < kChunks; ++q) {
+            const int x = lane + 32 * q;
+            if (x > kMPix) continue;
+            const __half h = __int2half_rn(v[q]);
+            px[y * 2 * kMPitch + x] = h;
+            if (x > 0) px[y * 2 * kMPitch + 2 * kMCopy + x - 1] = h;
         }
     }
+    __syncthreads();
+    // sum of squares of every candidate patch: running sums along rows, then columns
+    float *s_row = reinterpret_cast<float *>(s_list);  // [kMPix][kMCand], until the lists begin
+    constexpr int kSeg = 20;  // one segment a thread
+    static_assert(kMCand % kSeg == 0, "segments cover the window");
+    for (int i = threadIdx.x; i < kMPix * (kMCand / kSeg); i += kThreads) {
+        const int y = i % kMPix, x0 = (i / kMPix) * kSeg;
+        const __half *p = px + y * 2 * kMPitch + x0;
+        float sum = 0.f;
+        for (int q = 0; q < kPS - 1; ++q) sum += __half2float(p[q]) * __half2float(p[q]);
+        for (int q = 0; q < kSeg; ++q) {
+            const float in = __half2float(p[q + kPS - 1]), out = __half2float(p[q]);
+            sum += in * in;
+            s_row[y * kMCand + x0 + q] = sum;
+            sum -= out * out;
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kMCand * (kMCand / kSeg); i += kThreads) {
+        const int x = i % kMCand, y0 = (i / kMCand) * kSeg;
+        float sum = 0.f;
+        for (int q = 0; q < kPS - 1; ++q) sum += s_row[(y0 + q) * kMCand + x];
+        for (int q = 0; q < kSeg; ++q) {
+            sum += s_row[(y0 + q + kPS - 1) * kMCand + x];
+            s_sq[(y0 + q) * kMCand + x] = sum;
+            sum -= s_row[(y0 + q) * kMCand + x];
+        }
+    }
+    __syncthreads();
+
+    const int g = lane >> 2, t = lane & 3;
+    const int half = wid & 1, blk = wid >> 1;  // the pair of warps 2 blk, 2 blk + 1
+    // blocks beyond the last reference repeat it (their results are not written)
+    const int ri0 = bi + 4 * (blk / kMSide), rj0 = bj + 4 * (blk % kMSide);
+    const bool idle = ri0 >= nri || rj0 >= nrj;
+    const int ci0 = min(ri0, nri - 1), cj0 = min(rj0, nrj - 1);
+    MatchLane m;
+    m.t = t;
+    m.ly = ref_pos(ci0, H) - kHalfWin - oy;
+    m.lx = (ref_pos(cj0, W) - kHalfWin - ox) & ~1;
+    const int rx = ref_pos(min(rj0 + (g & 3), nrj - 1), W);
+    m.xlo = max(0, rx - kHalfWin) - ox;
+    m.xhi = min(W - kPS, rx + kHalfWin) - ox;
+    uint32_t own[2];  // window position of the references themselves
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int ry = ref_pos(min(ri0 + (g >> 2) + 2 * r, nri - 1), H);
+        m.ylo[r] = max(0, ry - kHalfWin) - oy - m.ly;
+        m.yhi[r] = min(H - kPS, ry + kHalfWin) - oy - m.ly;
+        const int ay = ry - oy, ax = rx - ox;
+        own[r] = (uint32_t)(ay * 128 + ax);
+        m.base[r] = s_sq[ay * kMCand + ax] + kMBias;
+        const uint32_t *p = s_px + ay * kMPitch + (ax & 1) * kMCopy + (ax >> 1) + t;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const __half2 v = __hmul2(*reinterpret_cast<const __half2 *>(p + (2 * k + h) * kMPitch),
+                                          __float2half2_rn(-2.f));
+                m.a[k][2 * h + r] = *reinterpret_cast<const uint32_t *>(&v);
+            }
+    }
+    m.all_lo = __reduce_max_sync(FULL, max(m.ylo[0], m.ylo[1]));
+    m.all_hi = __reduce_min_sync(FULL, min(m.yhi[0], m.yhi[1]));
+    const int any_lo = __reduce_min_sync(FULL, min(m.ylo[0], m.ylo[1]));
+    const int any_hi = __reduce_max_sync(FULL, max(m.yhi[0], m.yhi[1]));
+    const int bx = m.lx + g;
+    const uint32_t *bw = s_px + m.ly * kMPitch + (bx & 1) * kMCopy + (bx >> 1) + t;
+    uint32_t *list = s_list + wid * kMList + lane;
+    const uint32_t list_at = (uint32_t)__cvta_generic_to_shared(list);
+    uint32_t at[2] = {list_at, list_at + kMCap * 128};
+    float vt[2] = {0.f, 0.f};
+    float best[2][kMBest];
+#pragma unroll
+    for (int i = 0; i < 2 * kMBest; ++i) best[i / kMBest][i % kMBest] = kMFar;
+    if (!idle) match_scan<1>(m, half, kMFirst, kMFirst + 15, bw, s_sq, best, list, at, vt);
+#pragma unroll
+    for (int i = 0; i < 2 * kMBest; ++i) list[i * 32] = __float_as_uint(best[i / kMBest][i % kMBest]);
+    __syncthreads();
+    // warp `half` of the pair: the 16th smallest of the SSDs kept for its references
+    // (4 lanes x 2 warps x 6; floats above zero order like their bits), at most the
+    // threshold
+    if (!idle) {
+        const uint32_t *mine = s_list + 2 * blk * kMList + lane + half * kMBest * 32;
+        uint32_t k[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            k[i] = i < kMBest       ? mine[i * 32]
+                   : i < 2 * kMBest ? mine[kMList + (i - kMBest) * 32]
+                                    : kMNone;
+        sort16(k);
+        merge16(k, [&](int i) { return __shfl_xor_sync(FULL, k[i], 1); });
+        uint32_t top = 0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) top = max(top, min(k[i], __shfl_xor_sync(FULL, k[15 - i], 2)));
+        s_cnt[(2 * blk + half) * 64 + lane] =
+            min(top, __float_as_uint(kMBias + (float)thr));
+    }
+    __syncthreads();
+    if (!idle) {
+        vt[0] = __uint_as_float(s_cnt[2 * blk * 64 + lane]);
+        vt[1] = __uint_as_float(s_cnt[(2 * blk + 1) * 64 + lane]);
+        match_scan<2>(m, half, any_lo & ~3, any_hi, bw, s_sq, best, list, at, vt);
+    }
+    __syncwarp();
+    // the 16 smallest keys of each reference: a lane sorts its lists, the four lanes
+    // of a reference merge theirs, then the two warps
+    uint32_t k[16];
+    uint32_t *xch = s_list + wid * kMList;  // the warp's lists are its own until here
+    if (!idle) {
+        uint32_t mine[16];
+#pragma unroll 1
+        for (int r = 0; r < 2; ++r) {
+            const int n = (int)(at[r] - list_at) / 128 - r * kMCap;
+            const uint32_t *q = list + r * kMCap * 32;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) k[i] = i < n ? q[i * 32] : kMNone;
+            sort16(k);
+            for (int j = 16; __any_sync(FULL, j < n); ++j) {
+                uint32_t key = j < n ? q[j * 32] : kMNone;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) order(k[i], key);
+            }
+#pragma unroll
+            for (int x = 1; x <= 2; x *= 2) merge16(k, [&](int i) {
+                return __shfl_xor_sync(FULL, k[i], x);
+            });
+            if (r == half) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) mine[i] = k[i];
+            } else {  // for the other warp, over the first rows of list 0 or 1 (read above)
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (t == 0) xch[(r * kMCap + i) * 32 + g] = k[i];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) k[i] = mine[i];
+    }
+    __syncthreads();
+    if (idle) return;
+    const uint32_t *theirs = s_list + (wid ^ 1) * kMList + half * kMCap * 32 + g;
+    merge16(k, [&](int i) { return theirs[i * 32]; });
+    // drop the reference itself, if it is among them
+    const uint32_t self = half ? own[1] : own[0];
+    int cnt = 0;
+    bool past = false;
+#pragma unroll
+    for (int i = 0; i < 15; ++i) {
+        past = past || k[i] == self;
+        if (past) k[i] = k[i + 1];
+        cnt += k[i] != kMNone;
+    }
+    const int ri = ri0 + (g >> 2) + 2 * half, rj = rj0 + (g & 3);
+    if (ri >= nri || rj >= nrj) return;
+    const size_t o = (size_t)sl * nri * nrj + (size_t)ri * nrj + rj;
+    auto place = [&](int i) {  // entry i of the group: the reference, then the keys
+        if (i == 0) return ref_pos(ri, H) * W + ref_pos(rj, W);
+        const uint32_t key = k[i - 1];
+        return key == kMNone ? -1
+                             : (oy + (int)((key >> 7) & 63u)) * W + ox + (int)(key & 127u);
+    };
+    int *out = lists + o * kMaxGroup;
+#pragma unroll
+    for (int i = 0; i < kMaxGroup; ++i)
+        if (t == i / 4) out[i] = place(i);
+    if (t == 0) counts[o] = 1 + cnt;
 }
 
 // ---- collaborative filtering on the tensor cores ------------------------------
@@ -262,15 +593,6 @@ constexpr size_t kFootBytes = sizeof(float) * kFoot * kFootPitch;
 
 __device__ TcTables g_tc;
 __constant__ float c_k1[kPS];  // 1-D Kaiser window (K[a][b] = k1[a] k1[b])
-
-__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
-                                         uint32_t a3, uint32_t b0, uint32_t b1)
-{
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-        "{%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
 // x0 + x1 * 2^16-lane packing: hi = fp16 pair of (x0, x1), lo = fp16 pair of
 // the remainders (x - hi is exact in FP32).
@@ -1069,9 +1391,14 @@ cslsm_status match(const uint8_t *codes, int ns, int H, int W, int stage, int *l
     const long long total = (long long)ns * n_refs(H) * n_refs(W);
     if (total == 0) return CSLSM_OK;
     const int thr = kPS * kPS * (stage == 1 ? kTauHard : kTauWiener);
+    constexpr int kRefs = 4 * kMSide;
+    const long long blocks = (long long)((n_refs(W) + kRefs - 1) / kRefs) *
+                             ((n_refs(H) + kRefs - 1) / kRefs) * ns;  // < total < 2^31
+    CSLSM_CUDA(cudaFuncSetAttribute(bm3d_match_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kMSmem));
     LaunchScope ls(K_BM3D_MATCH, s);
-    bm3d_match_kernel<<<grid_for(total, kMatchWarps), kMatchWarps * 32, 0, s>>>(
-        codes, H, W, ns, thr, lists, counts, stop);
+    bm3d_match_kernel<<<(unsigned)blocks, kMWarps * 32, kMSmem, s>>>(codes, H, W, thr, lists,
+                                                                     counts, stop);
     CSLSM_LAUNCHED();
     return CSLSM_OK;
 }

@@ -69,6 +69,33 @@ def test_match_lists_bit_exact_outside_unit_range(cs, stage):
         np.testing.assert_array_equal(lists[z], idx)
 
 
+def _patterns(H, W):
+    """Slices on which the candidates' order, not their distance, decides: ties over whole
+    rows and columns, all matches in one tile column or row, full candidate lists."""
+    y, x = np.mgrid[:H, :W]
+    rng = np.random.default_rng(H * W)
+    noise = rng.random((H, W))
+    yield 0.3 + 0.02 * noise                  # few codes: many ties
+    yield (x >= W // 2) + 0.01 * noise        # vertical edge
+    yield 0.7 * (y >= H // 3) + 0.05 * noise  # horizontal edge
+    yield 0.4 * (x == W // 2)                 # one column
+    yield (x % 4 < 2).astype(float)           # stripes
+    yield ((x + y) % 5) / 5.0                 # diagonals
+
+
+# one reference, a few, one past a block of 4 x 4 and of 8 x 8, windows cut on every side
+@pytest.mark.parametrize("H,W", [(8, 9), (11, 46), (21, 33), (47, 48), (64, 35)])
+@pytest.mark.parametrize("stage", [1, 2])
+def test_match_lists_on_ties_and_edges(cs, H, W, stage):
+    img = np.stack(list(_patterns(H, W))).astype(np.float32)
+    lists, counts = cs.bm3d_match(to_dev(img), stage)
+    lists, counts = lists.cpu().numpy(), counts.cpu().numpy()
+    for z in range(len(img)):
+        idx, cnt = oracle.bm3d_match(img[z], stage)
+        np.testing.assert_array_equal(counts[z], cnt)
+        np.testing.assert_array_equal(lists[z], idx)
+
+
 def test_match_ties_on_constant_image(cs):
     img = np.full((1, 40, 44), 0.25, dtype=np.float32)
     lists, counts = cs.bm3d_match(to_dev(img), 1)
