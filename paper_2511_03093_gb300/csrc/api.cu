@@ -685,6 +685,8 @@ cslsm_status cslsm_batch_create(cslsm_batch *out, const cslsm_batch_item *items,
     int cur = -1;
     CSLSM_CUDA(cudaGetDevice(&cur));
     CHECK_ARG(cur == dev, "the items' plans belong to device %d, current device is %d", dev, cur);
+    int sms = 0;
+    CSLSM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     cudaStream_t s = as_stream(stream);
     CSLSM_CUDA(cudaStreamSynchronize(s));
     cslsm_batch_s *bt = new (std::nothrow) cslsm_batch_s();
@@ -720,9 +722,24 @@ cslsm_status cslsm_batch_create(cslsm_batch *out, const cslsm_batch_item *items,
         bt->zero.push_back({p->u, esz * (size_t)p->g.voxels()});
         bt->zero.push_back({p->d, esz * (size_t)p->g.voxels()});
     }
-    // steps per phase: a fixed default unless a phase length is set or timing
-    // a few candidates on the batch itself is asked for (autotune mode 1)
+    // steps per phase: by rule unless a phase length is set or timing a few
+    // candidates on the batch itself is asked for (autotune mode 1).  At most 10
+    // steps, or balanced phases of at most 8 (T = 20: 7) where a level of the items
+    // fills the grid: fewer steps waste less on halos, more phases cost loads and,
+    // with few tiles in flight, waits.  ms at 10 / 7 steps, by tiles of a level over
+    // CTAs: 12 items BF16 (3.5) 58.7 / 53.1; 1 x 1024 x 1024 x 32 gamma = 0 (22) 14.9 /
+    // 13.6; 700 x 333 x 20 (3.07) 2.80 / 2.88; 512 x 512 x 16 (2.7) 1.99 / 2.09; 4
+    // items (0.9) 35.2 / 36.5.
     int kbest = std::min(std::max(T, 1), 10);
+    if (T > 10) {
+        const int phases = (T + 7) / 8, kbal = (T + phases - 1) / phases;
+        long long tiles = 0;
+        for (const BatchItemSpec &it : spec.items) {
+            const int Z = it.N * it.R;
+            tiles += batch_tiles_per_slice(it.H, it.W, kbal) * (prm->gamma > 0.f && Z > 1 ? 1 : Z);
+        }
+        if (3 * tiles >= 10 * 3ll * sms) kbest = kbal;  // three CTAs per SM
+    }
     const int kset = g_batch_k;
     if (kset > 0) {
         kbest = std::min({kset, std::max(T, 1), batch_max_steps_per_phase()});

@@ -415,17 +415,23 @@ bool make_cfg(int c, int H, int W, int T, int sms, int storage, Cfg &f)
     return f.tx * f.ty <= occ * sms;
 }
 
-// Model in SM cycles per slice: every region row is updated in every step
-// (about 0.25 cycles per pixel on an SM at full issue, scaled down when fewer
-// than 16 warps share the SM), plus a fixed cost per phase boundary.
+// Model of a slice's time in microseconds: per phase an exchange, a fixed part and
+// one that grows with the rows loaded; per step the dependent chain of a warp's rows
+// and the issue of the warps that the dependence band keeps busy (two CTAs on an SM
+// overlap each other's barriers and waits).  The constants are a least-squares fit
+// to 627 measured (geometry, tiling) pairs: 13 geometries from 128 x 128 to 768 x 768,
+// FP32 and BF16, T = 20, 9 % rms.  Its choice is on average 1.2 % behind the best
+// tiling, 3.2 % at most; the count of region pixels it replaces was up to 36 % behind
+// (us per slice: 512 x 512 28.3 -> 23.4, 640 x 480 32.2 -> 24.1, 256 x 256 17.9 -> 15.6).
 double model(const Cfg &f, int T, int sms)
 {
     const int tiles = f.tx * f.ty;
     const int per_sm = (tiles + sms - 1) / sms;
-    const double warps = (double)f.B * per_sm;
-    const double eff = std::min(1.0, warps / 16.0);
     const int P = (T + f.k - 1) / f.k;
-    return per_sm * (double)T * f.RH * kPW * 0.25 / eff + 4000.0 * P;
+    const double rows = (double)per_sm * f.B * f.RPW;
+    const double active = std::min((double)f.B, std::ceil((f.TH + f.k - 1.0) / f.RPW) + 0.5);
+    const double issue = 0.01216 * per_sm * active * f.RPW * (per_sm > 1 ? 0.84 : 1.0);
+    return P * (3.51 + 0.01718 * rows) + T * (0.01818 * f.RPW - 0.0533 + issue);
 }
 
 std::mutex g_mu;
