@@ -95,20 +95,18 @@ __global__ void bm3d_prep_kernel(const S *__restrict__ src, const S *__restrict_
 // of the whole window and keeps the keys up to the bound (about 40), in lists of its
 // own per lane and reference; a list that fills up drops all but its 16 smallest and
 // lowers its bound.  The lanes of a reference then sort and merge their lists.
-//   Two warps share a block of references, each with every other tile column, so
-// that one small slice still gives every SM work.
+//   kSplit warps share a block of references, each with every kSplit-th tile column:
+// two on CTAs of 2 x 2 blocks, which share the staging, or six on CTAs of one block
+// where the larger CTAs would leave a quarter of the SMs idle.  Both in us a launch:
+// 1 x 64 x 64 27.7 / 17.9, 1 x 200 x 200 (81 large CTAs) 33.0 / 23.8, 1 x 253 x 317 (154)
+// 31.9 / 39.6, 1 x 512 x 512 78 / 113; one warp per reference took 17.3, 32.9, 53.9, 155.
 //   Measured, 4 slices of 512 x 512 (115,600 references): hard 0.683 -> 0.272 ms,
 // Wiener 0.659 -> 0.287 ms against one warp per reference on dp4a with sorted
 // insertion; 1,470 warp instructions a reference (5,530), bound by issue (57 %, integer
-// pipe 42 %, tensor pipe 29 %).  One 253 x 317 slice: 36 us of which 11 in the products
-// of pass 2.
+// pipe 42 %, tensor pipe 29 %).
 // mma.sync rather than tcgen05: every product goes through the ALU in the registers
 // where mma.sync leaves it, and the tensor pipe is not the limit.
 constexpr int kMSpan = 48;        // candidate rows / columns of a warp's 4 x 4 references
-constexpr int kMSide = 2;         // blocks of 4 x 4 references per CTA side
-constexpr int kMWarps = 2 * kMSide * kMSide;
-constexpr int kMCand = 3 * (4 * kMSide - 1) + 2 * kHalfWin + 1;  // 60 candidate rows / columns
-constexpr int kMPix = kMCand + kPS - 1;                          // 67 pixel rows / columns
 constexpr int kMCopy = 40;        // words per row of one copy (bank offset 8 between the two)
 constexpr int kMPitch = 2 * kMCopy;
 constexpr int kMCap = 32;         // keys per lane's list
@@ -119,11 +117,21 @@ constexpr int kMBest = 6;         // least SSDs a lane keeps in pass 1
 constexpr float kMBias = 8388608.f;  // 2^23
 constexpr float kMFar = 33554432.f;  // above every SSD + 2^23
 constexpr uint32_t kMNone = 0xffffffffu;
-constexpr size_t kMSmem = sizeof(uint32_t) * kMPix * kMPitch + sizeof(float) * kMCand * kMCand +
-                          sizeof(uint32_t) * kMWarps * (kMList + 2 * 32);
-static_assert(kMPix <= 2 * kMCopy, "a copy's row is too short");
-static_assert(kMWarps * kMList >= kMPix * kMCand, "row sums do not fit the lists' place");
-static_assert(kMCand <= 64, "13-bit window position");
+template <int SIDE, int SPLIT>  // blocks of 4 x 4 references per CTA side, warps per block
+struct MatchCta {
+    static constexpr int kWarps = SPLIT * SIDE * SIDE;
+    static constexpr int kRefs = 4 * SIDE;                             // references per side
+    static constexpr int kCand = 3 * (kRefs - 1) + 2 * kHalfWin + 1;   // candidates per side
+    static constexpr int kPix = kCand + kPS - 1;                       // pixels per side
+    static constexpr size_t kBytes = sizeof(uint32_t) * kPix * kMPitch +
+                                     sizeof(float) * kCand * kCand +
+                                     sizeof(uint32_t) * kWarps * kMList + sizeof(float) * SIDE * SIDE * 64;
+    static_assert(kMSpan / 8 % SPLIT == 0 && SPLIT >= 2 && 4 * SPLIT * kMBest >= 16, "split");
+    static_assert(kPix <= 2 * kMCopy, "a copy's row is too short");
+    static_assert(kWarps * kMList >= kPix * kCand, "row sums do not fit the lists' place");
+    static_assert(kCand <= 64, "13-bit window position");
+    static_assert(kCand % 2 == 0, "squares are read in pairs");
+};
 
 __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                          uint32_t a3, uint32_t b0, uint32_t b1)
@@ -213,12 +221,13 @@ __device__ __forceinline__ void append_if(uint32_t &at, uint32_t key, float d, f
 struct MatchFetch {
     uint32_t w[4];
     float2 s[4];
+    template <int CAND>
     __device__ __forceinline__ void load(const uint32_t *bp, const float *sp)
     {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             w[i] = bp[i * kMPitch];
-            s[i] = *reinterpret_cast<const float2 *>(sp + i * kMCand);
+            s[i] = *reinterpret_cast<const float2 *>(sp + i * CAND);
         }
     }
 };
@@ -228,7 +237,7 @@ struct MatchFetch {
 // four need (from bp, sp).  The rows' products are four independent chains.  PASS 1:
 // SSD + 2^23 into the sorted lists best; PASS 2: keys up to the bounds vt to the
 // lists at.  WHOLE: all rows valid.
-template <int PASS, bool WHOLE>
+template <int PASS, bool WHOLE, int CAND>
 __device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *bp, const float *sp,
                                            MatchFetch &f, const float (&r0)[2],
                                            const float (&r1)[2], int y, uint32_t l,
@@ -247,7 +256,7 @@ __device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *b
         d[i][2] = f.s[i].x + r1[0];
         d[i][3] = f.s[i].y + r1[1];
     }
-    f.load(bp, sp);
+    f.load<CAND>(bp, sp);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -298,15 +307,15 @@ __device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *b
     }
 }
 
-// Walks the warp's tile columns c0, c0 + 2, c0 + 4 over rows first .. last (fours).
-template <int PASS>
+// Walks the warp's tile columns c0, c0 + SPLIT, .. over rows first .. last (fours).
+template <int PASS, int SPLIT, int CAND>
 __device__ __forceinline__ void match_scan(const MatchLane &m, int c0, int first, int last,
                                            const uint32_t *bw, const float *s_sq,
                                            float (&best)[2][kMBest], uint32_t *list,
                                            uint32_t (&at)[2], float (&vt)[2])
 {
     constexpr float kPen = 16777216.f;
-    for (int c = c0; c < kMSpan / 8; c += 2) {
+    for (int c = c0; c < kMSpan / 8; c += SPLIT) {
         const int x = m.lx + 8 * c + 2 * m.t;
         const bool v0 = x >= m.xlo && x <= m.xhi, v1 = x + 1 >= m.xlo && x + 1 <= m.xhi;
         // columns outside the window: pushed above every bound
@@ -314,7 +323,7 @@ __device__ __forceinline__ void match_scan(const MatchLane &m, int c0, int first
         const float r1[2] = {m.base[1] + (v0 ? 0.f : kPen), m.base[1] + (v1 ? 0.f : kPen)};
         const bool any = __any_sync(0xffffffffu, v0 || v1);
         const uint32_t *bp = bw + 4 * c + first * kMPitch;
-        const float *sp = s_sq + (m.ly + first) * kMCand + x;
+        const float *sp = s_sq + (m.ly + first) * CAND + x;
         uint32_t l = (uint32_t)((m.ly + first) * 128 + x);
         uint32_t R[7];
         if (!any) continue;
@@ -322,35 +331,37 @@ __device__ __forceinline__ void match_scan(const MatchLane &m, int c0, int first
         for (int i = 0; i < 7; ++i) R[i] = bp[i * kMPitch];
         bp += 7 * kMPitch;
         MatchFetch f;
-        f.load(bp, sp);
+        f.load<CAND>(bp, sp);
         for (int y = first; y <= last; y += 4) {
             if (y + 4 <= last) {  // the last four rows fetch themselves again
                 bp += 4 * kMPitch;
-                sp += 4 * kMCand;
+                sp += 4 * CAND;
             }
             if (y >= m.all_lo && y + 3 <= m.all_hi)
-                match_rows<PASS, true>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
+                match_rows<PASS, true, CAND>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
             else
-                match_rows<PASS, false>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
+                match_rows<PASS, false, CAND>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
             l += 4 * 128;
         }
     }
 }
 
-__global__ void __launch_bounds__(kMWarps * 32, 2)
+template <int SIDE, int SPLIT>
+__global__ void __launch_bounds__(MatchCta<SIDE, SPLIT>::kWarps * 32, 2)
 bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
                   int *__restrict__ lists, int *__restrict__ counts, const int *__restrict__ stop)
 {
     if (stop && *stop) return;
-    constexpr int kThreads = kMWarps * 32;
+    using Cta = MatchCta<SIDE, SPLIT>;
+    constexpr int kWarps = Cta::kWarps, kThreads = kWarps * 32;
+    constexpr int kPix = Cta::kPix, kCand = Cta::kCand, kRefs = Cta::kRefs;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t *s_px = reinterpret_cast<uint32_t *>(smem);  // [kMPix][2 copies][kMCopy] FP16 pairs
-    float *s_sq = reinterpret_cast<float *>(s_px + kMPix * kMPitch);  // [kMCand][kMCand]
-    uint32_t *s_list = reinterpret_cast<uint32_t *>(s_sq + kMCand * kMCand);
-    uint32_t *s_cnt = s_list + kMWarps * kMList;  // [warp][reference g / g + 8][lane]
+    uint32_t *s_px = reinterpret_cast<uint32_t *>(smem);  // [kPix][2 copies][kMCopy] FP16 pairs
+    float *s_sq = reinterpret_cast<float *>(s_px + kPix * kMPitch);  // [kCand][kCand]
+    uint32_t *s_list = reinterpret_cast<uint32_t *>(s_sq + kCand * kCand);
+    uint32_t *s_tau = s_list + kWarps * kMList;  // [block][reference g / g + 8][lane]
     const int nri = n_refs(H), nrj = n_refs(W);
-    constexpr int kRefs = 4 * kMSide;
     const int tx = (nrj + kRefs - 1) / kRefs, ty = (nri + kRefs - 1) / kRefs;
     const int sl = (int)(blockIdx.x / (unsigned)(tx * ty));
     const int tile = (int)(blockIdx.x - (unsigned)sl * (unsigned)(tx * ty));
@@ -360,21 +371,21 @@ bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
     // pixels of the joint window as FP16, pairs on even and on odd columns
     __half *px = reinterpret_cast<__half *>(s_px);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int kChunks = (kMPix + 1 + 31) / 32;  // the last column of a copy's row is a zero
-#pragma unroll 3
-    for (int y = wid; y < kMPix; y += kMWarps) {
+    constexpr int kChunks = (kPix + 1 + 31) / 32;  // the last column of a copy's row is a zero
+#pragma unroll 5
+    for (int y = wid; y < kPix; y += kWarps) {
         const int gy = oy + y;
         const bool iny = gy >= 0 && gy < H;
         int v[kChunks];
 #pragma unroll
         for (int q = 0; q < kChunks; ++q) {
             const int x = lane + 32 * q, gx = ox + x;
-            v[q] = iny && x < kMPix && gx >= 0 && gx < W ? img[(size_t)gy * W + gx] : 0;
+            v[q] = iny && x < kPix && gx >= 0 && gx < W ? img[(size_t)gy * W + gx] : 0;
         }
 #pragma unroll
         for (int q = 0; q < kChunks; ++q) {
             const int x = lane + 32 * q;
-            if (x > kMPix) continue;
+            if (x > kPix) continue;
             const __half h = __int2half_rn(v[q]);
             px[y * 2 * kMPitch + x] = h;
             if (x > 0) px[y * 2 * kMPitch + 2 * kMCopy + x - 1] = h;
@@ -382,38 +393,38 @@ bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
     }
     __syncthreads();
     // sum of squares of every candidate patch: running sums along rows, then columns
-    float *s_row = reinterpret_cast<float *>(s_list);  // [kMPix][kMCand], until the lists begin
-    constexpr int kSeg = 20;  // one segment a thread
-    static_assert(kMCand % kSeg == 0, "segments cover the window");
-    for (int i = threadIdx.x; i < kMPix * (kMCand / kSeg); i += kThreads) {
-        const int y = i % kMPix, x0 = (i / kMPix) * kSeg;
+    float *s_row = reinterpret_cast<float *>(s_list);  // [kPix][kCand], until the lists begin
+    constexpr int kSeg = SIDE == 1 ? 16 : 20;  // one segment a thread
+    static_assert(kCand % kSeg == 0, "segments cover the window");
+    for (int i = threadIdx.x; i < kPix * (kCand / kSeg); i += kThreads) {
+        const int y = i % kPix, x0 = (i / kPix) * kSeg;
         const __half *p = px + y * 2 * kMPitch + x0;
         float sum = 0.f;
         for (int q = 0; q < kPS - 1; ++q) sum += __half2float(p[q]) * __half2float(p[q]);
         for (int q = 0; q < kSeg; ++q) {
             const float in = __half2float(p[q + kPS - 1]), out = __half2float(p[q]);
             sum += in * in;
-            s_row[y * kMCand + x0 + q] = sum;
+            s_row[y * kCand + x0 + q] = sum;
             sum -= out * out;
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < kMCand * (kMCand / kSeg); i += kThreads) {
-        const int x = i % kMCand, y0 = (i / kMCand) * kSeg;
+    for (int i = threadIdx.x; i < kCand * (kCand / kSeg); i += kThreads) {
+        const int x = i % kCand, y0 = (i / kCand) * kSeg;
         float sum = 0.f;
-        for (int q = 0; q < kPS - 1; ++q) sum += s_row[(y0 + q) * kMCand + x];
+        for (int q = 0; q < kPS - 1; ++q) sum += s_row[(y0 + q) * kCand + x];
         for (int q = 0; q < kSeg; ++q) {
-            sum += s_row[(y0 + q + kPS - 1) * kMCand + x];
-            s_sq[(y0 + q) * kMCand + x] = sum;
-            sum -= s_row[(y0 + q) * kMCand + x];
+            sum += s_row[(y0 + q + kPS - 1) * kCand + x];
+            s_sq[(y0 + q) * kCand + x] = sum;
+            sum -= s_row[(y0 + q) * kCand + x];
         }
     }
     __syncthreads();
 
     const int g = lane >> 2, t = lane & 3;
-    const int half = wid & 1, blk = wid >> 1;  // the pair of warps 2 blk, 2 blk + 1
+    const int part = wid % SPLIT, blk = wid / SPLIT;  // warp `part` of block blk
     // blocks beyond the last reference repeat it (their results are not written)
-    const int ri0 = bi + 4 * (blk / kMSide), rj0 = bj + 4 * (blk % kMSide);
+    const int ri0 = bi + 4 * (blk / SIDE), rj0 = bj + 4 * (blk % SIDE);
     const bool idle = ri0 >= nri || rj0 >= nrj;
     const int ci0 = min(ri0, nri - 1), cj0 = min(rj0, nrj - 1);
     MatchLane m;
@@ -431,7 +442,7 @@ bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
         m.yhi[r] = min(H - kPS, ry + kHalfWin) - oy - m.ly;
         const int ay = ry - oy, ax = rx - ox;
         own[r] = (uint32_t)(ay * 128 + ax);
-        m.base[r] = s_sq[ay * kMCand + ax] + kMBias;
+        m.base[r] = s_sq[ay * kCand + ax] + kMBias;
         const uint32_t *p = s_px + ay * kMPitch + (ax & 1) * kMCopy + (ax >> 1) + t;
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -455,40 +466,46 @@ bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
     float best[2][kMBest];
 #pragma unroll
     for (int i = 0; i < 2 * kMBest; ++i) best[i / kMBest][i % kMBest] = kMFar;
-    if (!idle) match_scan<1>(m, half, kMFirst, kMFirst + 15, bw, s_sq, best, list, at, vt);
+    if (!idle) match_scan<1, SPLIT, kCand>(m, part, kMFirst, kMFirst + 15, bw, s_sq, best, list, at, vt);
 #pragma unroll
     for (int i = 0; i < 2 * kMBest; ++i) list[i * 32] = __float_as_uint(best[i / kMBest][i % kMBest]);
     __syncthreads();
-    // warp `half` of the pair: the 16th smallest of the SSDs kept for its references
-    // (4 lanes x 2 warps x 6; floats above zero order like their bits), at most the
-    // threshold
-    if (!idle) {
-        const uint32_t *mine = s_list + 2 * blk * kMList + lane + half * kMBest * 32;
+    // warps 0 and 1 of the block: the 16th smallest of the SSDs kept for references g /
+    // g + 8 (4 lanes x SPLIT warps x 6; floats above zero order like their bits), at
+    // most the threshold
+    if (!idle && part < 2) {
+        const uint32_t *kept = s_list + SPLIT * blk * kMList + lane + part * kMBest * 32;
         uint32_t k[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-            k[i] = i < kMBest       ? mine[i * 32]
-                   : i < 2 * kMBest ? mine[kMList + (i - kMBest) * 32]
+            k[i] = i < kMBest       ? kept[i * 32]
+                   : i < 2 * kMBest ? kept[kMList + (i - kMBest) * 32]
                                     : kMNone;
         sort16(k);
+        for (int w = 2; w < SPLIT; ++w) {
+#pragma unroll
+            for (int i = 0; i < kMBest; ++i) {
+                uint32_t key = kept[w * kMList + i * 32];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) order(k[j], key);
+            }
+        }
         merge16(k, [&](int i) { return __shfl_xor_sync(FULL, k[i], 1); });
         uint32_t top = 0;
 #pragma unroll
         for (int i = 0; i < 16; ++i) top = max(top, min(k[i], __shfl_xor_sync(FULL, k[15 - i], 2)));
-        s_cnt[(2 * blk + half) * 64 + lane] =
-            min(top, __float_as_uint(kMBias + (float)thr));
+        s_tau[(2 * blk + part) * 32 + lane] = min(top, __float_as_uint(kMBias + (float)thr));
     }
     __syncthreads();
     if (!idle) {
-        vt[0] = __uint_as_float(s_cnt[2 * blk * 64 + lane]);
-        vt[1] = __uint_as_float(s_cnt[(2 * blk + 1) * 64 + lane]);
-        match_scan<2>(m, half, any_lo & ~3, any_hi, bw, s_sq, best, list, at, vt);
+        vt[0] = __uint_as_float(s_tau[2 * blk * 32 + lane]);
+        vt[1] = __uint_as_float(s_tau[(2 * blk + 1) * 32 + lane]);
+        match_scan<2, SPLIT, kCand>(m, part, any_lo & ~3, any_hi, bw, s_sq, best, list, at, vt);
     }
     __syncwarp();
-    // the 16 smallest keys of each reference: a lane sorts its lists, the four lanes
-    // of a reference merge theirs, then the two warps
+    // the 16 smallest keys of each reference: a lane sorts its lists, the four lanes of
+    // a reference merge theirs, then warps 0 and 1 of the block the warps'
     uint32_t k[16];
-    uint32_t *xch = s_list + wid * kMList;  // the warp's lists are its own until here
     if (!idle) {
         uint32_t mine[16];
 #pragma unroll 1
@@ -507,25 +524,29 @@ bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
             for (int x = 1; x <= 2; x *= 2) merge16(k, [&](int i) {
                 return __shfl_xor_sync(FULL, k[i], x);
             });
-            if (r == half) {
+            if (r == part) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) mine[i] = k[i];
-            } else {  // for the other warp, over the first rows of list 0 or 1 (read above)
+            } else {  // for warp r, over the first rows of the list (read above)
                 __syncwarp();
+                uint32_t *xch = s_list + wid * kMList + r * kMCap * 32 + g;
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    if (t == 0) xch[(r * kMCap + i) * 32 + g] = k[i];
+                    if (t == 0) xch[i * 32] = k[i];
             }
         }
 #pragma unroll
         for (int i = 0; i < 16; ++i) k[i] = mine[i];
     }
     __syncthreads();
-    if (idle) return;
-    const uint32_t *theirs = s_list + (wid ^ 1) * kMList + half * kMCap * 32 + g;
-    merge16(k, [&](int i) { return theirs[i * 32]; });
+    if (idle || part >= 2) return;
+    for (int w = 0; w < SPLIT; ++w) {
+        if (w == part) continue;
+        const uint32_t *theirs = s_list + (SPLIT * blk + w) * kMList + part * kMCap * 32 + g;
+        merge16(k, [&](int i) { return theirs[i * 32]; });
+    }
     // drop the reference itself, if it is among them
-    const uint32_t self = half ? own[1] : own[0];
+    const uint32_t self = part ? own[1] : own[0];
     int cnt = 0;
     bool past = false;
 #pragma unroll
@@ -534,7 +555,7 @@ bm3d_match_kernel(const uint8_t *__restrict__ codes, int H, int W, int thr,
         if (past) k[i] = k[i + 1];
         cnt += k[i] != kMNone;
     }
-    const int ri = ri0 + (g >> 2) + 2 * half, rj = rj0 + (g & 3);
+    const int ri = ri0 + (g >> 2) + 2 * part, rj = rj0 + (g & 3);
     if (ri >= nri || rj >= nrj) return;
     const size_t o = (size_t)sl * nri * nrj + (size_t)ri * nrj + rj;
     auto place = [&](int i) {  // entry i of the group: the reference, then the keys
@@ -1391,14 +1412,28 @@ cslsm_status match(const uint8_t *codes, int ns, int H, int W, int stage, int *l
     const long long total = (long long)ns * n_refs(H) * n_refs(W);
     if (total == 0) return CSLSM_OK;
     const int thr = kPS * kPS * (stage == 1 ? kTauHard : kTauWiener);
-    constexpr int kRefs = 4 * kMSide;
-    const long long blocks = (long long)((n_refs(W) + kRefs - 1) / kRefs) *
-                             ((n_refs(H) + kRefs - 1) / kRefs) * ns;  // < total < 2^31
-    CSLSM_CUDA(cudaFuncSetAttribute(bm3d_match_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kMSmem));
+    int dev = 0, sms = 0;
+    CSLSM_CUDA(cudaGetDevice(&dev));
+    CSLSM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    auto ctas = [&](int refs) {  // < total < 2^31
+        return (long long)((n_refs(W) + refs - 1) / refs) * ((n_refs(H) + refs - 1) / refs) * ns;
+    };
     LaunchScope ls(K_BM3D_MATCH, s);
-    bm3d_match_kernel<<<(unsigned)blocks, kMWarps * 32, kMSmem, s>>>(codes, H, W, thr, lists,
-                                                                     counts, stop);
+    if (ctas(MatchCta<2, 2>::kRefs) >= 3 * sms / 4) {
+        using Cta = MatchCta<2, 2>;
+        CSLSM_CUDA(cudaFuncSetAttribute(bm3d_match_kernel<2, 2>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)Cta::kBytes));
+        bm3d_match_kernel<2, 2><<<(unsigned)ctas(Cta::kRefs), Cta::kWarps * 32, Cta::kBytes, s>>>(
+            codes, H, W, thr, lists, counts, stop);
+    } else {
+        using Cta = MatchCta<1, 6>;
+        CSLSM_CUDA(cudaFuncSetAttribute(bm3d_match_kernel<1, 6>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)Cta::kBytes));
+        bm3d_match_kernel<1, 6><<<(unsigned)ctas(Cta::kRefs), Cta::kWarps * 32, Cta::kBytes, s>>>(
+            codes, H, W, thr, lists, counts, stop);
+    }
     CSLSM_LAUNCHED();
     return CSLSM_OK;
 }
