@@ -802,10 +802,12 @@ struct FilterArgs {
     float sigma;
     const int *stop;      // tolerance-stopped solve: skip (or nullptr)
     float *stat;          // [ns][nref] per-group kept count / sum W^2, or nullptr
+    int split;            // CTAs that share a block of references
 };
 
 // Persistent: each CTA takes 8 x 8 blocks of references (one slice each) in
-// turn, stages the block's footprint of g (and of the guide) in shared
+// turn, or a share of one where the blocks alone do not fill the GPU (one 253 x 317
+// slice: 143 blocks, two shares each, hard 68 -> 38 us, Wiener 86 -> 55 us), stages the block's footprint of g (and of the guide) in shared
 // memory, and its warps filter the block's groups one per warp.
 template <bool kWiener>
 __global__ void __launch_bounds__(kTcWarps * 32, 2) bm3d_filter_tc_kernel(const FilterArgs a)
@@ -831,7 +833,9 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bm3d_filter_tc_kernel(const 
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const float sigma = a.sigma, s2 = sigma * sigma, thr = kLambda3D * sigma;
-    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (long long work = blockIdx.x; work < ntiles * a.split; work += gridDim.x) {
+        const long long tile = work / a.split;
+        const int share = (int)(work - tile * a.split);
         const int sl = (int)(tile / ((long long)tbx * tby));
         const int rem = (int)(tile - (long long)sl * tbx * tby);
         const int bi = (rem / tbx) * kRefBlock, bj = (rem % tbx) * kRefBlock;
@@ -853,7 +857,7 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bm3d_filter_tc_kernel(const 
         __syncthreads();
         double *num = a.num + sl * HW, *wimg = a.wimg + sl * HW;
         const int nblk = (ei - bi + 1) * (ej - bj + 1);
-        for (int rr = wid; rr < nblk; rr += kTcWarps) {
+        for (int rr = share * kTcWarps + wid; rr < nblk; rr += kTcWarps * a.split) {
             const int r = (bi + rr / (ej - bj + 1)) * nrj + bj + rr % (ej - bj + 1);
             const size_t gi = (size_t)sl * nri * nrj + r;
             const int m = a.counts[gi];
@@ -969,6 +973,10 @@ __global__ void __launch_bounds__(kTcWarps * 32, 2) bm3d_filter_tc_kernel(const 
 // x_k = max(s_k - sigma^2 w_k, 0), w_k = c sqrt(m) / (sigma_hat_k + eps),
 // sigma_hat_k = sqrt(max(s_k^2 - 64 sigma^2, 0)); Xhat = Xc + mean.  Every
 // estimated patch is aggregated with weight 1 (FP64 sums; the counts are exact).
+// Bound by issue (71 %).  The partner's column comes over by one shuffle an element
+// that serves both the dot product and the rotation (two before), and the estimates
+// go out as FP64 reductions in L2, the counts as integers (FP64 compare-and-swap in
+// shared memory before): 4 x 256 x 256 2.33 -> 1.79 ms, the same bits.
 constexpr int kJacobiSweeps = 8;
 constexpr float kWnnmC = 2.8284271247461903f;  // 2 sqrt(2)
 
@@ -980,6 +988,7 @@ struct WnnmArgs {
     int H, W, ns;
     float sigma;
     const int *stop;
+    int split;           // CTAs that share a block of references
 };
 
 // Partner of column k in round r of the round robin over 16 columns.
@@ -996,7 +1005,7 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
 {
     if (a.stop && *a.stop) return;
     constexpr unsigned FULL = 0xffffffffu;
-    __shared__ double s_num[kFoot * kFootPitch], s_den[kFoot * kFootPitch];
+    __shared__ unsigned s_at[kFoot * kFootPitch];  // patches aggregated at each position
     __shared__ float s_n[kFoot * kFootPitch];
     __shared__ float s_mu[kFilterWarps][kPS * kPS];
     __shared__ float s_v[kFilterWarps][kMaxGroup][kMaxGroup + 1];  // [row l][column k]
@@ -1004,7 +1013,8 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
     const int H = a.H, W = a.W;
     const int nri = n_refs(H), nrj = n_refs(W);
     const int sl = blockIdx.z;
-    const int bi = blockIdx.y * kRefBlock, bj = blockIdx.x * kRefBlock;
+    const int share = (int)(blockIdx.x % (unsigned)a.split);
+    const int bi = blockIdx.y * kRefBlock, bj = (int)(blockIdx.x / (unsigned)a.split) * kRefBlock;
     const int ei = min(bi + kRefBlock, nri) - 1, ej = min(bj + kRefBlock, nrj) - 1;
     const int f0 = max(0, ref_pos(bi, H) - kHalfWin), f1 = min(H, ref_pos(ei, H) + kHalfWin + kPS);
     const int g0 = max(0, ref_pos(bj, W) - kHalfWin), g1 = min(W, ref_pos(ej, W) + kHalfWin + kPS);
@@ -1014,17 +1024,17 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
     for (int idx = threadIdx.x; idx < fh * fw; idx += blockDim.x) {
         const int y = idx / fw, x = idx - y * fw;
         const int l = y * kFootPitch + x;
-        s_num[l] = 0.0;
-        s_den[l] = 0.0;
+        s_at[l] = 0u;
         s_n[l] = noisy[(size_t)(f0 + y) * W + g0 + x];
     }
     __syncthreads();
 
+    double *num = a.num + sl * HW;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int k = lane >> 1, h = lane & 1;
+    const int k = lane >> 1, half = lane & 1;
     const float sigma = a.sigma, s2 = sigma * sigma;
     const int nblk = (ei - bi + 1) * (ej - bj + 1);
-    for (int rr = wid; rr < nblk; rr += kFilterWarps) {
+    for (int rr = share * kFilterWarps + wid; rr < nblk; rr += kFilterWarps * a.split) {
         const int r = (bi + rr / (ej - bj + 1)) * nrj + bj + rr % (ej - bj + 1);
         const size_t gi = (size_t)sl * nri * nrj + r;
         const int m = a.counts[gi];
@@ -1036,7 +1046,7 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
         for (int rw = 0; rw < 4; ++rw)
 #pragma unroll
             for (int c = 0; c < kPS; ++c)
-                x[rw * kPS + c] = act ? s_n[(py + 4 * h + rw) * kFootPitch + px + c] : 0.f;
+                x[rw * kPS + c] = act ? s_n[(py + 4 * half + rw) * kFootPitch + px + c] : 0.f;
         // the mean patch over the m active columns (butterfly over lanes of this half)
         const float inv_m = 1.f / (float)m;
 #pragma unroll
@@ -1047,23 +1057,25 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
             t += __shfl_xor_sync(FULL, t, 8);
             t += __shfl_xor_sync(FULL, t, 16);
             const float mu = t * inv_m;
-            if (k == 0) s_mu[wid][h * 4 * kPS + i] = mu;
+            if (k == 0) s_mu[wid][half * 4 * kPS + i] = mu;
             x[i] = act ? x[i] - mu : 0.f;
         }
-        // V = I: lane (k, h) holds V[8h + j][k]
+        // V = I: lane (k, h) holds V[8 half + j][k]
         float vc[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) vc[j] = (8 * h + j == k) ? 1.f : 0.f;
+        for (int j = 0; j < 8; ++j) vc[j] = (8 * half + j == k) ? 1.f : 0.f;
         for (int sw = 0; sw < kJacobiSweeps; ++sw) {
             for (int rd = 0; rd < 15; ++rd) {
                 const int p = rr_partner(k, rd);
-                const int src = 2 * p + h;
+                const int src = 2 * p + half;
+                // the partner's column, fetched once for the dot product and the rotation
+                float o[4 * kPS];
                 float own2 = 0.f, dot = 0.f;
 #pragma unroll
                 for (int i = 0; i < 4 * kPS; ++i) {
-                    const float o = __shfl_sync(FULL, x[i], src);
+                    o[i] = __shfl_sync(FULL, x[i], src);
                     own2 = fmaf(x[i], x[i], own2);
-                    dot = fmaf(x[i], o, dot);
+                    dot = fmaf(x[i], o[i], dot);
                 }
                 own2 += __shfl_xor_sync(FULL, own2, 1);
                 dot += __shfl_xor_sync(FULL, dot, 1);
@@ -1077,15 +1089,16 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
                     c = 1.f / sqrtf(1.f + t * t);
                     sn = c * t;
                 }
+                // lower column c x_lo - sn x_hi, higher sn x_lo + c x_hi, each as
+                // fma(f, x_lo, h x_hi): the two are rounded alike in both lanes
+                const float f = lo ? c : sn, h = lo ? -sn : c;
 #pragma unroll
-                for (int i = 0; i < 4 * kPS; ++i) {
-                    const float o = __shfl_sync(FULL, x[i], src);
-                    x[i] = lo ? c * x[i] - sn * o : sn * o + c * x[i];
-                }
+                for (int i = 0; i < 4 * kPS; ++i)
+                    x[i] = __fmaf_rn(f, lo ? x[i] : o[i], __fmul_rn(h, lo ? o[i] : x[i]));
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const float o = __shfl_sync(FULL, vc[j], src);
-                    vc[j] = lo ? c * vc[j] - sn * o : sn * o + c * vc[j];
+                    const float vo = __shfl_sync(FULL, vc[j], src);
+                    vc[j] = __fmaf_rn(f, lo ? vc[j] : vo, __fmul_rn(h, lo ? vo : vc[j]));
                 }
             }
         }
@@ -1098,9 +1111,9 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
         const float sh = sqrtf(fmaxf(nrm2 - 64.f * s2, 0.f));
         const float wk = kWnnmC * sqrtf((float)m) / (sh + 1e-8f);
         const float xk = fmaxf(sk - s2 * wk, 0.f);
-        if (h == 0) s_f[wid][k] = (act && sk > 0.f) ? xk / sk : 0.f;
+        if (half == 0) s_f[wid][k] = (act && sk > 0.f) ? xk / sk : 0.f;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) s_v[wid][8 * h + j][k] = vc[j];
+        for (int j = 0; j < 8; ++j) s_v[wid][8 * half + j][k] = vc[j];
         __syncwarp();
         // column k of Xc = sum_kk B[:, kk] f_kk V[k][kk]
         float o[4 * kPS];
@@ -1110,32 +1123,32 @@ __global__ void __launch_bounds__(kFilterWarps * 32, 2) wnnm_filter_kernel(const
             const float coef = s_f[wid][kk] * s_v[wid][k][kk];
 #pragma unroll
             for (int i = 0; i < 4 * kPS; ++i)
-                o[i] = fmaf(coef, __shfl_sync(FULL, x[i], 2 * kk + h), o[i]);
+                o[i] = fmaf(coef, __shfl_sync(FULL, x[i], 2 * kk + half), o[i]);
         }
+        // one FP64 reduction per estimated pixel, in L2; the counts as integers
         if (act) {
 #pragma unroll
             for (int rw = 0; rw < 4; ++rw)
 #pragma unroll
                 for (int c = 0; c < kPS; ++c) {
-                    const int l = (py + 4 * h + rw) * kFootPitch + px + c;
-                    const float est = o[rw * kPS + c] + s_mu[wid][h * 4 * kPS + rw * kPS + c];
-                    atomicAdd(&s_num[l], (double)est);
-                    atomicAdd(&s_den[l], 1.0);
+                    const float est = o[rw * kPS + c] + s_mu[wid][half * 4 * kPS + rw * kPS + c];
+                    red_add_f64(num + (size_t)(f0 + py + 4 * half + rw) * W + g0 + px + c, (double)est);
                 }
+            if (half == 0) atomicAdd(&s_at[py * kFootPitch + px], 1u);
         }
         __syncwarp();
     }
     __syncthreads();
-    double *num = a.num + sl * HW, *den = a.den + sl * HW;
+    // patches covering a pixel of the footprint: those at the 8 x 8 positions up and left
+    double *den = a.den + sl * HW;
     for (int idx = threadIdx.x; idx < fh * fw; idx += blockDim.x) {
         const int y = idx / fw, x = idx - y * fw;
-        const int l = y * kFootPitch + x;
-        const double d = s_den[l];
-        if (d != 0.0) {
-            const size_t o = (size_t)(f0 + y) * W + g0 + x;
-            atomicAdd(&num[o], s_num[l]);
-            atomicAdd(&den[o], d);
-        }
+        unsigned n = 0;
+        for (int dy = 0; dy < kPS; ++dy)
+#pragma unroll
+            for (int dx = 0; dx < kPS; ++dx)
+                if (dy <= y && dx <= x) n += s_at[(y - dy) * kFootPitch + x - dx];
+        if (n) red_add_f64(den + (size_t)(f0 + y) * W + g0 + x, (double)n);
     }
 }
 
@@ -1458,8 +1471,14 @@ cslsm_status launch_filter_tc(const FilterArgs &a, cudaStream_t s)
     CSLSM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const long long tiles = (long long)((n_refs(a.W) + kRefBlock - 1) / kRefBlock) *
                             ((n_refs(a.H) + kRefBlock - 1) / kRefBlock) * a.ns;
-    const unsigned grid = (unsigned)std::max(1ll, std::min(tiles, (long long)ps * sms));
-    bm3d_filter_tc_kernel<kWiener><<<grid, kTcWarps * 32, smem, s>>>(a);
+    // as many shares of a block as fit on the GPU at once, each at least a round of the
+    // CTA's warps (kRefBlock^2 groups, kTcWarps at a time)
+    FilterArgs b = a;
+    b.split = 1;
+    while (2 * b.split * kTcWarps <= kRefBlock * kRefBlock && 2 * b.split * tiles <= (long long)ps * sms)
+        b.split *= 2;
+    const unsigned grid = (unsigned)std::max(1ll, std::min(tiles * b.split, (long long)ps * sms));
+    bm3d_filter_tc_kernel<kWiener><<<grid, kTcWarps * 32, smem, s>>>(b);
     return CSLSM_OK;
 }
 
@@ -1467,7 +1486,7 @@ cslsm_status filter(int stage, const float *noisy, const float *guide, const Ws 
                     int H, int W, float sigma, cudaStream_t s, const int *stop = nullptr,
                     float *stat = nullptr)
 {
-    FilterArgs a{noisy, guide, w.lists, w.counts, w.num, w.den, H, W, ns, sigma, stop, stat};
+    FilterArgs a{noisy, guide, w.lists, w.counts, w.num, w.den, H, W, ns, sigma, stop, stat, 1};
     LaunchScope ls(K_BM3D_FILTER, s);
     cslsm_status e = stage == 1 ? launch_filter_tc<false>(a, s) : launch_filter_tc<true>(a, s);
     if (e) return e;
@@ -1506,9 +1525,16 @@ cslsm_status finish(double *num, double *den, S *out, const S *w, S *dual, uint8
 cslsm_status wnnm_filter(const float *noisy, const Ws &w, int ns, int H, int W, float sigma,
                          cudaStream_t s, const int *stop)
 {
-    WnnmArgs a{noisy, w.lists, w.counts, w.num, w.den, H, W, ns, sigma, stop};
-    const dim3 grid((n_refs(W) + kRefBlock - 1) / kRefBlock, (n_refs(H) + kRefBlock - 1) / kRefBlock,
-                    ns);
+    WnnmArgs a{noisy, w.lists, w.counts, w.num, w.den, H, W, ns, sigma, stop, 1};
+    const int tx = (n_refs(W) + kRefBlock - 1) / kRefBlock, ty = (n_refs(H) + kRefBlock - 1) / kRefBlock;
+    int dev = 0, sms = 0;
+    CSLSM_CUDA(cudaGetDevice(&dev));
+    CSLSM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // shares of a block as in launch_filter_tc (two CTAs per SM)
+    while (2 * a.split * kFilterWarps <= kRefBlock * kRefBlock &&
+           2ll * a.split * tx * ty * ns <= 2ll * sms)
+        a.split *= 2;
+    const dim3 grid(tx * a.split, ty, ns);
     LaunchScope ls(K_WNNM, s);
     wnnm_filter_kernel<<<grid, kFilterWarps * 32, 0, s>>>(a);
     CSLSM_LAUNCHED();
