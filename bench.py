@@ -813,9 +813,9 @@ def run_secondary(args) -> None:
         plan = cs.Plan(wk.H, wk.W, 1, wk.Z, torch.from_numpy(data["masks"]).to(dev))
         b = torch.from_numpy(data["b"]).to(dev)
         v = torch.empty((wk.Z, wk.H, wk.W), dtype=torch.float32, device=dev)
-        cs.set_autotune(1)
-        # TV: large slice-independent solves run as a one-item persistent batch
-        # (the library's route), the others as per-launch tiles
+        cs.set_autotune(4 if name.startswith("tv_tiles") else 1)  # 4: a forced tile variant
+        # TV: launches of a few steps each, or a one-item persistent batch (the
+        # library's route)
         doms = {"tikhonov": ("tikhonov_iter",), "tv": ("tv_tile", DOMINANT),
                 "bm3d": ("bm3d_match",)}[den]
         cs.timing_read(doms[0], reset=True)
@@ -838,7 +838,9 @@ def run_secondary(args) -> None:
                                                                         data["x"]))
         if den == "tikhonov":
             R = wk.Z
-            bytes_launch = vox * (16.0 + 8.0 / R)
+            # the streaming model of the iterations one launch runs (all of them when the
+            # solve keeps its pixel columns on chip: then `frac` compares, it does not bound)
+            bytes_launch = vox * (16.0 + 8.0 / R) * iters * steps / n_dom
             avg = ms_dom / n_dom / 1e3
             out["roofline"] = {"bound": "hbm", "kernel": dom, "achieved": bytes_launch / avg / 1e9,
                                "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -857,7 +859,7 @@ def run_secondary(args) -> None:
             out["path"] = "one-item persistent batch (cslsm_set_tv_route)"
         elif den == "tv":
             avg = ms_dom / n_dom / 1e3
-            fl = tv_flops_per_launch(wk.H, wk.W, 20) * wk.Z
+            fl = tv_flops_per_launch(wk.H, wk.W, 20) * wk.Z * iters * steps / n_dom
             out["roofline"] = {"bound": "alu", "kernel": dom, "achieved": fl / avg / 1e12,
                                "peak": alu_peak_tflops(2070.0), "unit": "TFLOP/s",
                                "frac": fl / avg / 1e12 / alu_peak_tflops(2070.0),

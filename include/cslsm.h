@@ -246,10 +246,13 @@ cslsm_status cslsm_batch_create(cslsm_batch *batch, const cslsm_batch_item *item
  * parameters and the alignment class of b and v_out stay the same (other b and
  * v_out are pointed to by a small copy on `stream`; recreating the batch
  * synchronises the device).
- *   mode 0 (default): the batch when one phase level holds at least 4 tiles
- *          per SM (large volumes), else the per-launch tiles; a batch that does
- *          not fit in device memory leaves the solve to the per-launch tiles;
- *   mode 1: always the per-launch tiles;   mode 2: always the batch.
+ *   mode 0 (default): the per-launch path, which runs the prox as a few launches
+ *          of several steps each (their exchange of the dual field, 16 bytes a
+ *          voxel up to 1 GB, belongs to the plan); the batch with BF16 state,
+ *          or beyond that size, when one phase level holds at least 4 tiles per
+ *          SM (large volumes); a batch that does not fit in device memory
+ *          leaves the solve to the per-launch path;
+ *   mode 1: always the per-launch path;   mode 2: always the batch.
  * On the batch path a non-NULL stats makes the call synchronise `stream` and
  * report a device-side wait that ran out (CSLSM_ERR_TIMEOUT).  Returns
  * CSLSM_ERR_INVALID_ARG for other modes. */
@@ -384,7 +387,9 @@ int cslsm_abi_version(void);
 
 /* TV prox tile shapes (process-wide setting).  The TV kernel comes in four
  * variants (column chunks x row bands) with a tile shape chosen per launch
- * geometry.  mode 0 (default): shapes from a cost model of the work per SM.
+ * geometry; it runs where the phase launches (see cslsm_set_tv_route) do not:
+ * under stream capture before their exchange exists, beyond its size, and when
+ * forced.  mode 0 (default): shapes from a cost model of the work per SM.
  * mode 1: on the first launch of each (device, H, W, steps, slices) key that
  * is not being captured into a CUDA graph, time every variant on the actual
  * launch (three runs each; the prox is idempotent, so this only costs time)
@@ -393,7 +398,7 @@ int cslsm_abi_version(void);
  * mode clears the kept choices. */
 cslsm_status cslsm_set_autotune(int mode);
 
-/* The TV tile shape a prox launch of this geometry would use now (on the
+/* The shape a tile-kernel prox launch of this geometry would use now (on the
  * current device): shape4 (host int[4]) = {variant, tile rows, tile columns,
  * region rows}.  steps <= 24 (longer proxes run in chunks). */
 cslsm_status cslsm_tv_shape(int H, int W, int steps, int nslices, int *shape4);

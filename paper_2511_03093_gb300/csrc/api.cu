@@ -277,8 +277,9 @@ namespace {
 // A TV solve whose prox is slice-independent (gamma = 0 or Z = 1), with a fixed
 // iteration count from u = d = 0 in the plan's own state, can run as a one-item
 // persistent batch (the same bits as the per-launch tiles, which recompute a
-// halo of T + 1 pixels in every launch).  Auto mode takes that path when one
-// phase level holds enough tiles to fill the GPU twice over.
+// halo of T + 1 pixels, or its phases).  Auto mode takes that path when one phase
+// level holds enough tiles to fill the GPU twice over and the phase launches are not
+// the faster ones.
 bool tv_route_applies(const cslsm_plan_s *plan, const cslsm_admm_params *prm, float gam,
                       bool use_tol, const void *u_io)
 {
@@ -288,6 +289,11 @@ bool tv_route_applies(const cslsm_plan_s *plan, const cslsm_admm_params *prm, fl
         prm->init_user || u_io != nullptr || prm->iters < 1)
         return false;
     if (mode == 2) return true;
+    // the phase launches are faster but with BF16 state (1024 x 1024 x 32: 1,413 us an
+    // iteration here, 1,541 there; FP32 1,350 / 1,221, FP16 512 x 512 x 16 194 / 185)
+    if (prm->storage != CSLSM_STORE_BF16 && tv_get_mode() <= 1 &&
+        tv_phases_fit(plan->g.H, plan->g.W, plan->g.Z()))
+        return false;
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -382,16 +388,35 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
     const int *stop = use_tol ? reinterpret_cast<const int *>(plan->tol) : nullptr;  // .stop
     int checks = 0;
     const bool tv = prm->denoiser == CSLSM_DEN_TV;
-    if (tv && prm->lambda > 0.f && prm->tv_inner > tv_max_steps_per_launch()) {
-        const size_t need = 4 * (gam > 0.f ? 1 : (size_t)g.Z()) * (size_t)g.HW();
-        if (plan->pbuf_floats < need) {
-            CSLSM_CUDA(cudaStreamSynchronize(s));
-            cudaFree(plan->pbuf);
-            plan->pbuf = nullptr;
-            plan->pbuf_floats = 0;
-            CSLSM_CUDA(cudaMalloc(&plan->pbuf, sizeof(float) * need));
-            plan->pbuf_floats = need;
+    // the dual-field exchange of proxes of nslices slices at a time: required for long
+    // proxes, otherwise only wanted (not allocated under stream capture, nor insisted on)
+    auto reserve_pbuf = [&](int nslices) -> cslsm_status {
+        if (!(prm->lambda > 0.f)) return CSLSM_OK;
+        const size_t need = tv_pbuf_floats(g.H, g.W, prm->tv_inner, nslices);
+        if (plan->pbuf_floats >= need) return CSLSM_OK;
+        const bool must = prm->tv_inner > tv_max_steps_per_launch();
+        if (!must) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            CSLSM_CUDA(cudaStreamIsCapturing(s, &cap));
+            if (cap != cudaStreamCaptureStatusNone) return CSLSM_OK;
         }
+        CSLSM_CUDA(cudaStreamSynchronize(s));
+        cudaFree(plan->pbuf);
+        plan->pbuf = nullptr;
+        plan->pbuf_floats = 0;
+        const cudaError_t e = cudaMalloc(&plan->pbuf, sizeof(float) * need);
+        if (e == cudaErrorMemoryAllocation && !must) {
+            cudaGetLastError();
+            plan->pbuf = nullptr;
+            return CSLSM_OK;
+        }
+        CSLSM_CUDA(e);
+        plan->pbuf_floats = need;
+        return CSLSM_OK;
+    };
+    if (tv && prm->lambda > 0.f && (gam == 0.f || prm->tv_inner > tv_max_steps_per_launch())) {
+        st = reserve_pbuf(gam > 0.f ? 1 : g.Z());
+        if (st) return st;
     }
     const bool patchwise = prm->denoiser == CSLSM_DEN_BM3D || prm->denoiser == CSLSM_DEN_WNNM;
     if (patchwise) {
@@ -474,7 +499,7 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
             if (gam == 0.f) {
                 a.n0 = 0;
                 a.nslices = g.Z();
-                st = tv_prox_slices(a, plan->pbuf, s);
+                st = tv_prox_slices(a, plan->pbuf, plan->pbuf_floats, s);
                 if (st) return st;
             } else {
                 a.n0 = 0;
@@ -493,9 +518,11 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
                 }
                 if (!swept) {
                     a.nslices = 1;
+                    st = reserve_pbuf(1);
+                    if (st) return st;
                     for (int n = 0; n < g.Z(); ++n) {
                         a.n0 = n;
-                        st = tv_prox_slices(a, plan->pbuf, s);
+                        st = tv_prox_slices(a, plan->pbuf, plan->pbuf_floats, s);
                         if (st) return st;
                     }
                 }
@@ -598,9 +625,20 @@ cslsm_status cslsm_denoise(int denoiser, const float *in, float *out, int Z, int
     a.tau = prm->tv_tau;
     a.T = prm->tv_inner;
     float *pbuf = nullptr;
-    if (a.theta > 0.f && a.T > tv_max_steps_per_launch())
-        CSLSM_CUDA(cudaMallocAsync(&pbuf, sizeof(float) * 4 * nv, s));
-    st = tv_prox_slices(a, pbuf, s);
+    size_t need = a.theta > 0.f ? tv_pbuf_floats(H, W, a.T, Z) : 0;
+    if (need && a.T <= tv_max_steps_per_launch()) {  // wanted, not needed
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CSLSM_CUDA(cudaStreamIsCapturing(s, &cap));
+        if (cap != cudaStreamCaptureStatusNone ||
+            cudaMallocAsync(&pbuf, sizeof(float) * need, s) != cudaSuccess) {
+            cudaGetLastError();
+            pbuf = nullptr;
+            need = 0;
+        }
+    } else if (need) {
+        CSLSM_CUDA(cudaMallocAsync(&pbuf, sizeof(float) * need, s));
+    }
+    st = tv_prox_slices(a, pbuf, need, s);
     if (pbuf) cudaFreeAsync(pbuf, s);
     return st;
 }

@@ -134,7 +134,12 @@ struct TvSlices {
 // Chambolle TV prox of every listed slice.  Uses the plan-provided dual
 // buffers pbuf (4 * nslices * H * W floats) only when T exceeds the largest
 // step count one launch covers; pbuf may be nullptr otherwise.
-cslsm_status tv_prox_slices(const TvSlices &a, float *pbuf, cudaStream_t s);
+cslsm_status tv_prox_slices(const TvSlices &a, float *pbuf, size_t pbuf_floats, cudaStream_t s);
+// Floats of the dual-field exchange that a prox of this geometry wants (on the current
+// device; more than tv_max_steps_per_launch() steps need it, others run without).
+size_t tv_pbuf_floats(int H, int W, int T, int nslices);
+// Whether that exchange is small enough for the prox to run in phases of a few steps.
+bool tv_phases_fit(int H, int W, int nslices);
 int tv_max_steps_per_launch();
 // 0: tile shapes from the cost model; 1: time the kernel variants on the first
 // launch of every shape key (outside stream capture) and keep the fastest;

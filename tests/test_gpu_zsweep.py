@@ -122,3 +122,35 @@ def test_wait_timeout_is_reported_and_recovers(cs):
     for r, g_ in zip(ref, again):
         assert torch.equal(r, g_)
     plan.close()
+
+
+# a region larger than the image, one pixel past a tile, odd widths (no paired accesses),
+# steps for one to several launches, slice by slice (gamma > 0) and all slices at once
+@pytest.mark.parametrize("Z,H,W", [(1, 1, 3), (2, 19, 41), (3, 44, 40), (2, 45, 83), (4, 130, 97),
+                                   (8, 256, 192)])
+@pytest.mark.parametrize("T", [1, 3, 20, 24])
+@pytest.mark.parametrize("gamma", [0.0, 0.25])
+@pytest.mark.parametrize("storage", ["fp32", "bf16", "fp16"])
+def test_phase_launches_match_tiles_bitwise(cs, Z, H, W, T, gamma, storage):
+    masks, b = _problem(Z + H + W + T, 1, Z, H, W)
+    plan = cs.Plan(H, W, 1, Z, masks)
+    prm = cs.Params(rho=1.0, lam=0.05, gamma=gamma, iters=2, denoiser="tv", tv_inner=T,
+                    storage=storage)
+    cs.zsweep_config(False)
+    cs.set_tv_route(1)
+    out = []
+    for mode in (0, 4):  # the default launches, the tile kernel
+        cs.set_autotune(mode)
+        u, d = (torch.empty(plan.vol_shape, dtype=cs.STORAGE_DTYPE[storage], device="cuda")
+                for _ in range(2))
+        v = plan.solve(b, prm, u=u, d=d)
+        out.append((v.cpu(), u.float().cpu(), d.float().cpu()))
+    x = torch.rand(Z, H, W, generator=torch.Generator().manual_seed(3)).cuda()
+    tiles = cs.denoise(x, prm)
+    cs.set_autotune(0)
+    assert torch.equal(cs.denoise(x, prm), tiles)
+    cs.set_tv_route(0)
+    cs.zsweep_config(True)
+    for a, e in zip(*out):
+        assert torch.equal(a, e)
+    plan.close()
