@@ -373,6 +373,17 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
         if (st != CSLSM_ERR_OOM || g_tv_route.load() == 2) return st;
         cudaGetLastError();  // the failed allocation's (non-sticky) error
     }
+    if (prm->denoiser == CSLSM_DEN_TIKHONOV && !use_tol && prm->iters >= 1 &&
+        tikhonov_solve_applies(g)) {
+        st = launch_tikhonov_solve(g, masks_of(plan), store, u_io, d_io, prm->init_user != 0, b,
+                                   prm->rho, prm->lambda, gam, prm->iters, v_out, s);
+        if (st) return st;
+        if (stats) {
+            stats->iters_done = prm->iters;
+            stats->rel_change = -1.0;
+        }
+        return CSLSM_OK;
+    }
     if (!prm->init_user) {
         CSLSM_CUDA(cudaMemsetAsync(u, 0, esz * nv, s));
         CSLSM_CUDA(cudaMemsetAsync(d, 0, esz * nv, s));

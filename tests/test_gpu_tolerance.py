@@ -72,3 +72,31 @@ def test_iteration_count_matches_oracle(cs, iters, tol):
         rel = np.linalg.norm(to_np(v) - v_r) / np.linalg.norm(v_r)
         assert rel <= 1e-4
     plan.close()
+
+
+# one plane, both sides of the sizes the one-launch solve is compiled for, an odd pixel count
+@pytest.mark.parametrize("Z", [1, 2, 7, 8, 9, 16, 17, 31, 32])
+@pytest.mark.parametrize("gamma", [0.0, 0.2])
+@pytest.mark.parametrize("storage", ["fp32", "bf16", "fp16"])
+def test_one_launch_tikhonov_equals_iteration_launches(cs, Z, gamma, storage):
+    """A tolerance that is never met runs one launch per iteration: the same bits, state too."""
+    H, W = 37, 53
+    g = torch.Generator().manual_seed(Z)
+    masks = (torch.rand(Z, H, W, generator=g) < 0.5).to(torch.uint8).cuda()
+    b = torch.rand(1, H, W, generator=g).cuda()
+    u0, d0 = (torch.rand(Z, H, W, generator=g).to(cs.STORAGE_DTYPE[storage]) for _ in range(2))
+    plan = cs.Plan(H, W, 1, Z, masks)
+    out = []
+    for tol in (0.0, 1e-30):
+        prm = cs.Params(rho=0.9, lam=0.05, gamma=gamma, iters=7, denoiser="tikhonov", tol=tol,
+                        check_every=100, storage=storage)
+        for init in (False, True):
+            u, d = u0.cuda(), d0.cuda()
+            v = plan.solve(b, prm, u=u, d=d, init_user=init)
+            out.append((v.cpu(), u.float().cpu(), d.float().cpu()))
+        out.append((plan.solve(b, prm).cpu(),))
+    for a, e in zip(out[:3], out[3:]):
+        for x, y in zip(a, e):
+            assert torch.equal(x, y)
+    assert torch.equal(out[2][0], out[0][0])
+    plan.close()
