@@ -14,12 +14,10 @@
 //  - Matching: the inner products of 4 x 4 references with their joint window by
 //    mma.sync, the selection on integer keys (see the matching section).  Bit-exact.
 //  - Filtering on the tensor cores, one warp per group (see its section).
-//    A CTA owns an 8x8 block of references: it stages g (and the basic
-//    estimate) of the block's footprint in shared memory and aggregates the
-//    block's estimates there with shared atomics before one global atomic
-//    flush per footprint pixel.  Numerators and denominators accumulate in
-//    FP64, so the order of the atomics changes sums only at the 1e-16 level and
-//    repeated calls give the same FP32 result.
+//    A CTA stages g (and the basic estimate) of the footprint of an 8x8 block of
+//    references in shared memory and filters the block or a share of it.
+//  - Aggregation by FP64 reductions in L2, so the order of the sums shows only at the
+//    1e-16 level and repeated calls give the same FP32 result.
 #include <cuda_runtime.h>
 
 #include <cmath>
