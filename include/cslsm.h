@@ -309,7 +309,7 @@ cslsm_status cslsm_batch_destroy(cslsm_batch batch);
  * gradients) and writes dL/dlogits and scalar_bar (device double[3]) =
  * {dL/drho, dL/dlambda, dL/dgamma} for the given v_bar = dL/dv^K.
  * keep_duals = 1 trades memory for time: the segment recompute keeps every
- * slice's prox input and its tv_steps + 1 dual iterates, so the reverse sweep
+ * slice's prox input and its recorded dual steps, so the reverse sweep
  * reads them instead of recomputing them (same results bit for bit).  The
  * workspace then grows by ckpt_every x Z x (2 tv_steps + 3) x B x H x W
  * floats (29 GB for batch 8 x 512 x 512 x 16, 20 steps, checkpoints every 5
