@@ -476,7 +476,7 @@ struct HuberRing {
     {
 #pragma unroll
         for (int i = 0; i < RPW; ++i)  // outside the image any valid address (nothing is read)
-            src[i] = rec + (size_t)first * step + ((in0 >> i) & 1u ? t.off(i, a.g.W) : 0);
+            src[i] = rec + (size_t)max(first, 0) * step + ((in0 >> i) & 1u ? t.off(i, a.g.W) : 0);
     }
     // Fetches the rows of the next step (going down) as one group of copies into
     // slot `slot`; an empty group when there is none.
@@ -644,9 +644,10 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
     } else {
         // pbar^T = theta grad ubar; hbar = ubar; -<ubar, div p^T>
         const float *ub = a.Ubar + bi * a.g.NV();
-        const float *r = rec + (size_t)(a.T - 1) * a.g.B * 2 * HW;
-        auto proj = [&](int gi, float2 &x1, float2 &x2) {  // p^T of a row
-            const bool i0 = gi >= 0 && gi < H && t.in0, i1 = gi >= 0 && gi < H && t.in1;
+        const float *r = rec + (size_t)max(a.T - 1, 0) * a.g.B * 2 * HW;
+        auto proj = [&](int gi, float2 &x1, float2 &x2) {  // p^T of a row (p^0 = 0)
+            const bool in = a.T > 0 && gi >= 0 && gi < H;
+            const bool i0 = in && t.in0, i1 = in && t.in1;
             x1 = ld_pair(r, gi * W + t.gc, i0, i1, a.pair);
             x2 = ld_pair(r + HW, gi * W + t.gc, i0, i1, a.pair);
             const float2 sc = huber_scale(x1, x2);
@@ -817,6 +818,8 @@ struct Prm {
     float rho, lam, gam, tau, eps;
     int K, T, S;
     float theta() const { return lam / (rho + 2.f * gam); }
+    // dual steps of a prox: none where theta underflows to 0 (the prox is the identity)
+    int steps() const { return theta() > 0.f ? T : 0; }
 };
 
 inline dim3 pgrid(const Geo &g) { return dim3((unsigned)((g.HW() + kT - 1) / kT), g.B); }
@@ -870,8 +873,8 @@ HuberShape huber_shape(const Geo &g, int T, bool reverse)
         else if (huber_tiles(g, 2, 7) >= 152) h = {2, 7};
         else h = {2, 10};
     }
-    const int P = (T + h.k - 1) / h.k;  // balanced phases
-    h.k = (T + P - 1) / P;
+    const int P = std::max(1, (T + h.k - 1) / h.k);  // balanced phases
+    h.k = std::max(1, (T + P - 1) / P);
     return h;
 }
 
@@ -919,11 +922,11 @@ HuberArgs huber_args(const Geo &g, const Prm &P, int k, bool pair)
     a.rho = P.rho;
     a.gam = P.gam;
     a.theta = P.theta();
-    a.inv_theta = 1.f / a.theta;
+    a.inv_theta = a.theta > 0.f ? 1.f / a.theta : 0.f;
     a.tau = P.tau;
     a.eps = P.eps;
-    a.kappa = P.eps / a.theta;
-    a.T = P.T;
+    a.kappa = a.theta > 0.f ? P.eps / a.theta : 0.f;
+    a.T = P.steps();
     a.hh = k + 1;
     a.hc = a.hh + (a.hh & 1);
     a.pair = pair;
@@ -937,7 +940,8 @@ cslsm_status slice_prox(const Geo &g, const Prm &P, const float *Wn, const float
                         const float *C, float *Hb, float *Pa, float *Pb, float *rec, float *Un,
                         float *Dn, bool pair, cudaStream_t s)
 {
-    const HuberShape sh = huber_shape(g, P.T, false);
+    const int T = P.steps();
+    const HuberShape sh = huber_shape(g, T, false);
     HuberArgs a = huber_args(g, P, sh.k, pair);
     a.Wn = Wn;
     a.A = A;
@@ -945,9 +949,9 @@ cslsm_status slice_prox(const Geo &g, const Prm &P, const float *Wn, const float
     a.Hb = Hb;
     const size_t hw2 = (size_t)g.B * 2 * g.HW();
     float *out = Pa;
-    for (int t = 0; t < P.T; t += sh.k) {
-        a.ns = std::min(sh.k, P.T - t);
-        const bool last = t + a.ns == P.T;
+    for (int t = 0; t == 0 || t < T; t += sh.k) {
+        a.ns = std::min(sh.k, T - t);
+        const bool last = t + a.ns == T;
         a.Pout = last ? nullptr : out;
         a.rec = rec ? rec + (size_t)t * hw2 : nullptr;
         a.Un = last ? Un : nullptr;
@@ -966,7 +970,8 @@ cslsm_status slice_prox_bwd(const Geo &g, const Prm &P, const float *Wn, const f
                             float *Pa, float *Pb, float *Wbar, float *Abar, float *Cbar,
                             double *acc, bool pair, cudaStream_t s)
 {
-    const HuberShape sh = huber_shape(g, P.T, true);
+    const int T = P.steps();
+    const HuberShape sh = huber_shape(g, T, true);
     HuberArgs a = huber_args(g, P, sh.k, pair);
     a.Wn = Wn;
     a.A = A;
@@ -980,7 +985,7 @@ cslsm_status slice_prox_bwd(const Geo &g, const Prm &P, const float *Wn, const f
     a.Cbar = Cbar;
     a.acc = acc;
     float *out = Pa;
-    for (int t = P.T; t > 0; t -= sh.k) {
+    for (int t = T; t == T || t > 0; t -= sh.k) {
         a.ns = std::min(sh.k, t);
         a.t0 = t - a.ns;
         a.Pout = a.t0 > 0 ? out : nullptr;

@@ -83,6 +83,29 @@ def test_tiled_dual_steps_match_fp64_oracle(cs, B, Z, H, W, T):
     assert rel_l2(lg.grad.cpu().numpy(), lg64.grad.numpy()) <= 1e-3
 
 
+@pytest.mark.parametrize("Z", [1, 3])
+@pytest.mark.parametrize("keep", [False, True])
+def test_theta_that_underflows_leaves_the_prox_out(cs, Z, keep):
+    """lambda / (rho + 2 gamma) rounds to 0: u = h, as the oracle gives without dual steps."""
+    logits, b, _ = _problem(31 + Z, 2, Z, 19, 22)
+    vbar = torch.randn(2, Z, 19, 22, generator=torch.Generator().manual_seed(15))
+    lg = logits.cuda().requires_grad_(True)
+    r, l_, gm = _scalars(rho=4.0, lam=1e-45)
+    v = cs.unrolled_admm(lg, b.cuda(), r, l_, gm, keep_duals=keep, **CFG)
+    (v * vbar.cuda()).sum().backward()
+    lg64 = logits.double().requires_grad_(True)
+    r64, l64, g64 = _scalars(rho=4.0, lam=1e-45, dev="cpu", dtype=torch.float64)
+    v64 = un.unrolled_admm(lg64, b.double(), r64, l64, g64, iters=CFG["iters"], T=0,
+                           tau=CFG["tv_tau"], eps=CFG["huber_eps"])
+    (v64 * vbar.double()).sum().backward()
+    assert rel_l2(v.detach().cpu().numpy(), v64.detach().numpy()) <= 1e-5
+    assert rel_l2(lg.grad.cpu().numpy(), lg64.grad.numpy()) <= 1e-3
+    for p, p64 in ((r, r64), (gm, g64)):
+        e = float(p64.grad)
+        assert abs(float(p.grad) - e) <= 1e-3 * max(abs(e), 1e-3)
+    assert float(l_.grad) == 0.0
+
+
 def test_checkpoint_period_does_not_change_gradients(cs):
     logits, b, _ = _problem(5, 1, 4, 20, 18)
     vbar = torch.randn(1, 4, 20, 18, generator=torch.Generator().manual_seed(6)).cuda()
