@@ -438,9 +438,11 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
             plan->bm3d_ws = nullptr;
             plan->bm3d_ws_bytes = 0;
             CSLSM_CUDA(cudaMalloc(&plan->bm3d_ws, need));
-            CSLSM_CUDA(cudaMemsetAsync(plan->bm3d_ws, 0, need, s));
             plan->bm3d_ws_bytes = need;
         }
+        // the sums of one slice lie where another call had the images of all of them
+        st = bm3d_clear(plan->bm3d_ws, gam > 0.f ? 1 : g.Z(), g.H, g.W, s);
+        if (st) return st;
     }
     const Masks m = masks_of(plan);
     int k = 0;

@@ -199,9 +199,11 @@ struct Bm3dSlices {
     const int *stop = nullptr;  // device flag of a tolerance-stopped solve: skip when set
 };
 int bm3d_nref(int H, int W);
-// Device workspace for nslices slices; it must be zero-filled before its first
-// use (the accumulators are cleared again by every call).
+// Device workspace for nslices slices.  Its accumulators must be zero (bm3d_clear)
+// before the first call on nslices slices, and are zero again after every call; a
+// workspace that other sizes have used in between is cleared again.
 size_t bm3d_workspace_bytes(int nslices, int H, int W);
+cslsm_status bm3d_clear(void *ws, int nslices, int H, int W, cudaStream_t s);
 cslsm_status bm3d_slices(const Bm3dSlices &b, void *ws, cudaStream_t s);
 // WNNM u-step on the same groups and workspace (hard-stage matching, one pass).
 cslsm_status wnnm_slices(const Bm3dSlices &b, void *ws, cudaStream_t s);

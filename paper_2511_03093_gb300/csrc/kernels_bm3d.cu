@@ -1608,6 +1608,13 @@ size_t bm3d_workspace_bytes(int ns, int H, int W)
            al(ns * nref * kMaxGroup * sizeof(int)) + al(ns * nref * sizeof(int)) + 256;
 }
 
+cslsm_status bm3d_clear(void *ws, int ns, int H, int W, cudaStream_t s)
+{
+    const size_t HW = (size_t)H * W;
+    CSLSM_CUDA(cudaMemsetAsync(carve(ws, ns, H, W).num, 0, 2 * al(ns * HW * sizeof(double)), s));
+    return CSLSM_OK;
+}
+
 cslsm_status wnnm_slices(const Bm3dSlices &b, void *ws, cudaStream_t s)
 {
     cslsm_status e = upload_constants();

@@ -211,3 +211,23 @@ def test_full_run_bm3d(cs, gamma):
     p_gpu, p_ref = oracle.psnr(to_np(v), data["x"]), oracle.psnr(v_r, data["x"])
     assert abs(p_gpu - p_ref) <= DPSNR, (p_gpu, p_ref)
     plan.close()
+
+
+@pytest.mark.parametrize("denoiser", ["bm3d", "wnnm"])
+def test_slice_solve_after_volume_solve_on_one_plan(cs, denoiser):
+    """gamma > 0 (one slice at a time) after gamma = 0 (all slices at once): the workspace's
+    layouts differ, so the slice's sums lie where the volume's images were."""
+    w = synth.Workload("ws", 5, 40, 36, mask_p=0.5, seed=41, n_blobs=40)
+    data = synth.generate(w)
+    b = to_dev(100.0 * data["b"])
+
+    def solve(plan, gamma):
+        prm = cs.Params(rho=1.0, lam=0.0, gamma=gamma, iters=2, denoiser=denoiser,
+                        bm3d_sigma=5.0)
+        return to_np(plan.solve(b, prm))
+
+    plans = [cs.Plan(w.H, w.W, 1, w.Z, to_dev(data["masks"])) for _ in range(2)]
+    solve(plans[0], 0.0)
+    assert rel_l2(solve(plans[0], 0.3), solve(plans[1], 0.3)) <= 1e-6
+    for p in plans:
+        p.close()
