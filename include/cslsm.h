@@ -79,7 +79,9 @@ typedef enum {
  *                 every kernel after the check that met the tolerance returns
  *                 at once; the call synchronises `stream` once at its end to
  *                 report the outcome.
- *                 0 runs exactly `iters` iterations without synchronising.
+ *                 0 runs exactly `iters` iterations without synchronising (with
+ *                 gamma > 0 TV synchronises once at the end to report a wait that
+ *                 ran out, except while `stream` is being captured).
  *   check_every   >= 1, used only when tol > 0.
  *   denoiser      a cslsm_denoiser.
  *   tv_inner      TV: Chambolle steps per prox (>= 1).
@@ -118,7 +120,13 @@ typedef struct cslsm_plan_s *cslsm_plan;
  *   masks     device uint8, [R][H][W] if per_slice == 0 or [Z][H][W] if 1.
  * The plan packs the patterns into one R-bit word per pixel and shot (bit r
  * = mirror open for plane r; diag(Phi Phi^T) is its popcount, Sec. III-B) and
- * allocates its workspace (about 3 * Z*H*W floats).  Synchronises `stream`. */
+ * allocates its workspace (about 3 * Z*H*W floats).  Synchronises `stream`.
+ * A plan's first solve of a kind allocates what that kind needs besides, and the
+ * plan keeps it (no buffer is freed before the plan is): TV 16 bytes a voxel
+ * with gamma = 0 (1 GB at most unless tv_inner > 24), or 16 to 32 bytes a pixel of
+ * one slice with gamma > 0;
+ * BM3D and WNNM about 45 bytes a voxel, or a pixel with gamma > 0; tol > 0 one more
+ * volume of floats. */
 cslsm_status cslsm_plan_create(cslsm_plan *plan, int H, int W, int n_shots, int R,
                                const uint8_t *masks, int per_slice, void *stream);
 
@@ -151,7 +159,12 @@ cslsm_status cslsm_adjoint(cslsm_plan plan, const float *b, float *v, void *stre
  *           resume a solve; when NULL the plan's own state buffers are used
  *           (then init_user must be 0).
  *   stats   host, optional.
- * v_out must not overlap u_io, d_io or b. */
+ * v_out must not overlap u_io, d_io or b.
+ * A solve with tol = 0 may be captured into a CUDA graph once the same kind of solve
+ * has run on the plan (so that nothing is left to allocate), and replayed as long as
+ * the plan and the caller's buffers live, whatever else the plan solves between
+ * replays.  A capture on a fresh plan is refused where the solve must allocate; TV
+ * with tv_inner <= 24 and gamma = 0 then runs each prox in one launch instead. */
 cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_params *params,
                               float *v_out, void *u_io, void *d_io, cslsm_admm_stats *stats,
                               void *stream);

@@ -42,13 +42,14 @@ struct cslsm_plan_s {
     int nsets = 0;
     float *u = nullptr, *d = nullptr, *w = nullptr;  // [Z][H][W] state and workspace
     float *vprev = nullptr;                          // [Z][H][W], tolerance checks only
-    float *pbuf = nullptr;                           // TV dual buffers for long proxes
+    float *pbuf = nullptr;                           // TV dual-field exchange
     size_t pbuf_floats = 0;
+    std::vector<void *> outgrown;  // smaller buffers that a captured solve may still use
     double *partials = nullptr;  // reduction partials (2 doubles per block)
     int npartials = 0;
     double *red_out = nullptr;  // 2 doubles
     TolState *tol = nullptr;    // device-side stopping state of tolerance solves
-    void *bm3d_ws = nullptr;     // BM3D workspace (zero-filled on allocation)
+    void *bm3d_ws = nullptr;     // BM3D / WNNM workspace
     size_t bm3d_ws_bytes = 0;
     ZsweepWs zs;                 // persistent z sweep (TV, gamma > 0)
     // slice-independent TV solves run as a one-item persistent batch, kept while
@@ -139,12 +140,33 @@ void free_plan(cslsm_plan_s *p)
     cudaFree(p->w);
     cudaFree(p->vprev);
     cudaFree(p->pbuf);
+    for (void *q : p->outgrown) cudaFree(q);
     zsweep_release(p->zs);
     cudaFree(p->partials);
     cudaFree(p->red_out);
     cudaFree(p->tol);
     cudaFree(p->bm3d_ws);
     delete p;
+}
+
+// A larger buffer in place of *buf.  The smaller one stays allocated until the plan is
+// destroyed: work in flight or a CUDA graph captured from an earlier solve may use it
+// (a plan's buffers have two sizes, one slice's and all slices').  Another stream or
+// thread may be capturing; an allocation here does not concern its capture.
+cudaError_t grow(cslsm_plan_s *p, void **buf, size_t bytes)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    void *q = nullptr;
+    const cudaError_t e = cudaMalloc(&q, bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+    }
+    if (*buf) p->outgrown.push_back(*buf);
+    *buf = q;
+    return cudaSuccess;
 }
 
 cslsm_status pack(cslsm_plan_s *p, const uint8_t *masks, int per_slice, cudaStream_t s)
@@ -280,8 +302,9 @@ namespace {
 // halo of T + 1 pixels, or its phases).  Auto mode takes that path when one phase
 // level holds enough tiles to fill the GPU twice over and the phase launches are not
 // the faster ones.
+// `phases`: the phase launches can run (they have, or may still get, their exchange).
 bool tv_route_applies(const cslsm_plan_s *plan, const cslsm_admm_params *prm, float gam,
-                      bool use_tol, const void *u_io)
+                      bool use_tol, const void *u_io, bool phases)
 {
     const int mode = g_tv_route.load();
     if (mode == 1) return false;
@@ -291,7 +314,7 @@ bool tv_route_applies(const cslsm_plan_s *plan, const cslsm_admm_params *prm, fl
     if (mode == 2) return true;
     // the phase launches are faster but with BF16 state (1024 x 1024 x 32: 1,413 us an
     // iteration here, 1,541 there; FP32 1,350 / 1,221, FP16 512 x 512 x 16 194 / 185)
-    if (prm->storage != CSLSM_STORE_BF16 && tv_get_mode() <= 1 &&
+    if (phases && prm->storage != CSLSM_STORE_BF16 && tv_get_mode() <= 1 &&
         tv_phases_fit(plan->g.H, plan->g.W, plan->g.Z()))
         return false;
     int dev = 0, sms = 0;
@@ -366,7 +389,37 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
     const size_t esz = store == CSLSM_STORE_FP32 ? 4 : 2;
     const float gam = g.Z() > 1 ? prm->gamma : 0.f;
     const bool use_tol = prm->tol > 0.f;
-    if (tv_route_applies(plan, prm, gam, use_tol, u_io)) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CSLSM_CUDA(cudaStreamIsCapturing(s, &cap));
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    // the dual-field exchange of proxes of nslices slices at a time: required for long
+    // proxes, otherwise only wanted (not allocated under stream capture, nor insisted on)
+    auto reserve_pbuf = [&](int nslices) -> cslsm_status {
+        const size_t need = tv_pbuf_floats(g.H, g.W, prm->tv_inner, nslices);
+        if (plan->pbuf_floats >= need) return CSLSM_OK;
+        const bool must = prm->tv_inner > tv_max_steps_per_launch();
+        if (capturing) {
+            if (!must) return CSLSM_OK;
+            set_error("TV with %d steps allocates on its first solve: run one before capturing",
+                      prm->tv_inner);
+            return CSLSM_ERR_CUDA;
+        }
+        void *buf = plan->pbuf;
+        const cudaError_t e = grow(plan, &buf, sizeof(float) * need);
+        if (e == cudaErrorMemoryAllocation && !must) return CSLSM_OK;
+        CSLSM_CUDA(e);
+        plan->pbuf = (float *)buf;
+        plan->pbuf_floats = need;
+        return CSLSM_OK;
+    };
+    bool route = tv_route_applies(plan, prm, gam, use_tol, u_io, true);
+    if (!route && prm->denoiser == CSLSM_DEN_TV && prm->lambda > 0.f && gam == 0.f) {
+        st = reserve_pbuf(g.Z());
+        if (st) return st;
+        if (!capturing && plan->pbuf_floats < tv_pbuf_floats(g.H, g.W, prm->tv_inner, g.Z()))
+            route = tv_route_applies(plan, prm, gam, use_tol, u_io, false);
+    }
+    if (route) {
         st = routed_tv_solve(plan, b, prm, v_out, stats, s);
         // auto mode: a batch that does not fit (memory) leaves the solve to the
         // per-launch tiles; a forced batch reports it
@@ -399,45 +452,19 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
     const int *stop = use_tol ? reinterpret_cast<const int *>(plan->tol) : nullptr;  // .stop
     int checks = 0;
     const bool tv = prm->denoiser == CSLSM_DEN_TV;
-    // the dual-field exchange of proxes of nslices slices at a time: required for long
-    // proxes, otherwise only wanted (not allocated under stream capture, nor insisted on)
-    auto reserve_pbuf = [&](int nslices) -> cslsm_status {
-        if (!(prm->lambda > 0.f)) return CSLSM_OK;
-        const size_t need = tv_pbuf_floats(g.H, g.W, prm->tv_inner, nslices);
-        if (plan->pbuf_floats >= need) return CSLSM_OK;
-        const bool must = prm->tv_inner > tv_max_steps_per_launch();
-        if (!must) {
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            CSLSM_CUDA(cudaStreamIsCapturing(s, &cap));
-            if (cap != cudaStreamCaptureStatusNone) return CSLSM_OK;
-        }
-        CSLSM_CUDA(cudaStreamSynchronize(s));
-        cudaFree(plan->pbuf);
-        plan->pbuf = nullptr;
-        plan->pbuf_floats = 0;
-        const cudaError_t e = cudaMalloc(&plan->pbuf, sizeof(float) * need);
-        if (e == cudaErrorMemoryAllocation && !must) {
-            cudaGetLastError();
-            plan->pbuf = nullptr;
-            return CSLSM_OK;
-        }
-        CSLSM_CUDA(e);
-        plan->pbuf_floats = need;
-        return CSLSM_OK;
-    };
-    if (tv && prm->lambda > 0.f && (gam == 0.f || prm->tv_inner > tv_max_steps_per_launch())) {
-        st = reserve_pbuf(gam > 0.f ? 1 : g.Z());
+    if (tv && prm->lambda > 0.f && gam > 0.f && prm->tv_inner > tv_max_steps_per_launch()) {
+        st = reserve_pbuf(1);
         if (st) return st;
     }
     const bool patchwise = prm->denoiser == CSLSM_DEN_BM3D || prm->denoiser == CSLSM_DEN_WNNM;
     if (patchwise) {
         const size_t need = bm3d_workspace_bytes(gam > 0.f ? 1 : g.Z(), g.H, g.W);
         if (plan->bm3d_ws_bytes < need) {
-            CSLSM_CUDA(cudaStreamSynchronize(s));
-            cudaFree(plan->bm3d_ws);
-            plan->bm3d_ws = nullptr;
-            plan->bm3d_ws_bytes = 0;
-            CSLSM_CUDA(cudaMalloc(&plan->bm3d_ws, need));
+            if (capturing) {
+                set_error("BM3D and WNNM allocate on a plan's first solve: run one before capturing");
+                return CSLSM_ERR_CUDA;
+            }
+            CSLSM_CUDA(grow(plan, &plan->bm3d_ws, need));
             plan->bm3d_ws_bytes = need;
         }
         // the sums of one slice lie where another call had the images of all of them
@@ -448,7 +475,7 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
     int k = 0;
     double rel = -1.0;
     bool stopped = false;
-    bool used_zsweep = false;
+    bool used_zsweep = false, asked = false;
     for (k = 0; k < prm->iters; ++k) {
         const bool last = (k == prm->iters - 1);
         const bool check = use_tol && k > 0 && ((k + 1) % prm->check_every == 0 || last);
@@ -531,8 +558,11 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
                 }
                 if (!swept) {
                     a.nslices = 1;
-                    st = reserve_pbuf(1);
-                    if (st) return st;
+                    if (!asked && a.theta > 0.f) {
+                        st = reserve_pbuf(1);
+                        if (st) return st;
+                        asked = true;
+                    }
                     for (int n = 0; n < g.Z(); ++n) {
                         a.n0 = n;
                         st = tv_prox_slices(a, plan->pbuf, plan->pbuf_floats, s);

@@ -1,0 +1,64 @@
+"""Solves captured into a CUDA graph: replays give the solve's own bits, whatever the plan
+did in between."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cs():
+    from paper_2511_03093_gb300 import build as b
+
+    b.build()
+    import paper_2511_03093_gb300 as m
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    return m
+
+
+def _problem(cs, seed, Z, H, W):
+    g = torch.Generator().manual_seed(seed)
+    masks = (torch.rand(Z, H, W, generator=g) < 0.5).to(torch.uint8).cuda()
+    return cs.Plan(H, W, 1, Z, masks), (torch.rand(1, H, W, generator=g) * Z / 2).cuda()
+
+
+def _capture(plan, b, prm, v):
+    """A graph of one solve into v (the plan has run the same solve before)."""
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        plan.solve(b, prm, v_out=v)
+    return graph
+
+
+def _replay(graph, v):
+    v.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    return v.cpu()
+
+
+@pytest.mark.parametrize("denoiser,tv_inner", [("tv", 20), ("tv", 30), ("bm3d", 1), ("wnnm", 1)])
+def test_replay_after_a_solve_that_needs_more_memory(cs, denoiser, tv_inner):
+    """gamma > 0, slice by slice, is captured with the plan's small buffers; gamma = 0 needs
+    larger ones.  The replay still finds its own."""
+    plan, b = _problem(cs, 3, 6, 64, 72)
+    small, large = (cs.Params(rho=1.0, lam=0.05, gamma=g, iters=3, denoiser=denoiser,
+                              tv_inner=tv_inner) for g in (0.3, 0.0))
+    cs.zsweep_config(False)
+    try:
+        v = torch.empty(plan.vol_shape, device="cuda")
+        want = plan.solve(b, small, v_out=v).cpu()
+        graph = _capture(plan, b, small, v)
+        other = plan.solve(b, large).cpu()
+        junk = torch.full((1 << 20,), 3.0, device="cuda")  # takes memory that was given back
+        for _ in range(2):
+            assert torch.equal(_replay(graph, v), want)
+        assert torch.equal(plan.solve(b, large).cpu(), other)
+        del junk
+    finally:
+        cs.zsweep_config(True)
+        torch.cuda.synchronize()
+        plan.close()
