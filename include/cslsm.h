@@ -264,8 +264,9 @@ cslsm_status cslsm_batch_create(cslsm_batch *batch, const cslsm_batch_item *item
  *          voxel up to 1 GB, belongs to the plan); the batch with BF16 state,
  *          or beyond that size, when one phase level holds at least 4 tiles per
  *          SM (large volumes); a batch that does not fit in device memory
- *          leaves the solve to the per-launch path;
- *   mode 1: always the per-launch path;   mode 2: always the batch.
+ *          leaves the solve to the per-launch path, and so does stream capture;
+ *   mode 1: always the per-launch path;   mode 2: always the batch (a capture
+ *          returns CSLSM_ERR_UNSUPPORTED).
  * On the batch path a non-NULL stats makes the call synchronise `stream` and
  * report a device-side wait that ran out (CSLSM_ERR_TIMEOUT).  Returns
  * CSLSM_ERR_INVALID_ARG for other modes. */

@@ -412,7 +412,13 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
         plan->pbuf_floats = need;
         return CSLSM_OK;
     };
-    bool route = tv_route_applies(plan, prm, gam, use_tol, u_io, true);
+    // (the batch is re-pointed by copies from the host at the time of the call, which a
+    // graph would repeat with whatever stands there then: not under capture)
+    bool route = !capturing && tv_route_applies(plan, prm, gam, use_tol, u_io, true);
+    if (capturing && g_tv_route.load() == 2 && tv_route_applies(plan, prm, gam, use_tol, u_io, true)) {
+        set_error("a solve on the batch route cannot be captured");
+        return CSLSM_ERR_UNSUPPORTED;
+    }
     if (!route && prm->denoiser == CSLSM_DEN_TV && prm->lambda > 0.f && gam == 0.f) {
         st = reserve_pbuf(g.Z());
         if (st) return st;

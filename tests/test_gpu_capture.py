@@ -62,3 +62,26 @@ def test_replay_after_a_solve_that_needs_more_memory(cs, denoiser, tv_inner):
         cs.zsweep_config(True)
         torch.cuda.synchronize()
         plan.close()
+
+
+def test_capture_where_the_batch_route_applies(cs):
+    """BF16 state and many tiles: the solve runs as a persistent batch, its capture as launches
+    of the same bits; a forced batch refuses the capture."""
+    plan, b = _problem(cs, 5, 16, 512, 512)
+    prm = cs.Params(rho=1.0, lam=0.05, iters=2, denoiser="tv", tv_inner=20, storage="bf16")
+    v = torch.empty(plan.vol_shape, device="cuda")
+    want = plan.solve(b, prm, v_out=v).cpu()
+    graph = _capture(plan, b, prm, v)
+    for _ in range(2):
+        assert torch.equal(_replay(graph, v), want)
+    cs.set_tv_route(2)
+    try:
+        assert torch.equal(plan.solve(b, prm).cpu(), want)
+        with pytest.raises(cs.CslsmError) as e:
+            _capture(plan, b, prm, v)
+        assert e.value.status == 4
+    finally:
+        cs.set_tv_route(0)
+    torch.cuda.synchronize()
+    assert torch.equal(plan.solve(b, prm).cpu(), want)
+    plan.close()
