@@ -485,7 +485,16 @@ cslsm_status launch(const TvSlices &s, const Cfg &f, ZsweepWs &ws, void *u, void
         a.stall = g_stall;
     }
     a.stop = s.stop;
-    a.base = ws.next_base;
+    // Epoch ids go on from launch to launch, so the flags that launches before left are
+    // below this launch's.  A graph repeats a captured launch's ids, which its own replay
+    // before would then satisfy: there the flags are cleared first and the ids start
+    // at 0, below every id that a later launch outside the graph uses.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CSLSM_CUDA(cudaStreamIsCapturing(st, &cap));
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    if (capturing)
+        CSLSM_CUDA(cudaMemsetAsync(ws.flags, 0, sizeof(unsigned) * f.tx * f.ty, st));
+    a.base = capturing ? 0u : ws.next_base;
     ws.next_base += (unsigned)(a.Z * a.P);
 
     cudaLaunchConfig_t cfg{};

@@ -85,3 +85,23 @@ def test_capture_where_the_batch_route_applies(cs):
     torch.cuda.synchronize()
     assert torch.equal(plan.solve(b, prm).cpu(), want)
     plan.close()
+
+
+@pytest.mark.parametrize("Z,H,W", [(2, 40, 36), (6, 200, 200), (5, 255, 257)])
+@pytest.mark.parametrize("storage", ["fp32", "bf16"])
+def test_replays_of_the_z_sweep(cs, Z, H, W, storage):
+    """The sweep's tiles wait for one another by epoch ids: a replay must not be satisfied by
+    the ids of the one before, nor a later solve by a replay's."""
+    plan, b = _problem(cs, Z + H, Z, H, W)
+    prm, other = (cs.Params(rho=1.0, lam=0.05, gamma=0.3, iters=4, denoiser="tv", tv_inner=t,
+                            storage=storage) for t in (20, 7))
+    v = torch.empty(plan.vol_shape, device="cuda")
+    want = plan.solve(b, prm, v_out=v).cpu()
+    want_other = plan.solve(b, other).cpu()
+    graph = _capture(plan, b, prm, v)
+    for _ in range(5):
+        assert torch.equal(_replay(graph, v), want)
+        assert torch.equal(plan.solve(b, other).cpu(), want_other)
+        assert torch.equal(_replay(graph, v), want)
+    assert torch.equal(plan.solve(b, prm).cpu(), want)
+    plan.close()
