@@ -144,7 +144,8 @@ cslsm_status tv_prox_slices(const TvSlices &a, float *pbuf, size_t pbuf_floats, 
 // Floats of the dual-field exchange that a prox of this geometry wants (on the current
 // device; more than tv_max_steps_per_launch() steps need it, others run without).
 size_t tv_pbuf_floats(int H, int W, int T, int nslices);
-// Whether that exchange is small enough for the prox to run in phases of a few steps.
+// Whether the prox can run in phases of a few steps: the exchange is small enough and the
+// slices fit a grid.
 bool tv_phases_fit(int H, int W, int nslices);
 int tv_max_steps_per_launch();
 // 0: tile shapes from the cost model; 1: time the kernel variants on the first

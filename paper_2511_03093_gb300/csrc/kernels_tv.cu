@@ -414,6 +414,7 @@ cslsm_status choose_shape(const TvLaunch &a, int dev, int sms, cudaStream_t st, 
 
 // The exchange of p (16 bytes a voxel) is kept to 1 GB; larger volumes run elsewhere.
 constexpr size_t kPhaseMaxFloats = 256ull << 20;
+constexpr int kPhaseMaxSlices = 65535;  // a grid's y extent; more slices run elsewhere too
 
 struct PhaseShape {
     int rpw = 0, P = 0, k = 0, hh = 0, hc = 0, TH = 0, TW = 0, tx = 0, ty = 0;
@@ -556,7 +557,10 @@ cslsm_status tv_query_shape(int H, int W, int T, int nslices, int *out4)
     return CSLSM_OK;
 }
 
-bool tv_phases_fit(int H, int W, int nslices) { return 4ull * nslices * H * W <= kPhaseMaxFloats; }
+bool tv_phases_fit(int H, int W, int nslices)
+{
+    return nslices <= kPhaseMaxSlices && 4ull * nslices * H * W <= kPhaseMaxFloats;
+}
 
 int tv_get_mode()
 {
@@ -576,7 +580,9 @@ size_t tv_pbuf_floats(int H, int W, int T, int nslices)
     const size_t all = 4ull * nslices * H * W;
     if (T > kMaxSteps) return all;
     int dev = 0, sms = 0;
-    if (tv_get_mode() > 1 || T < 1 || all > kPhaseMaxFloats || device_info(dev, sms) != CSLSM_OK) return 0;
+    if (tv_get_mode() > 1 || T < 1 || !tv_phases_fit(H, W, nslices) ||
+        device_info(dev, sms) != CSLSM_OK)
+        return 0;
     return phase_best(H, W, T, nslices, sms).P > 1 ? all : 0;
 }
 
@@ -585,7 +591,7 @@ cslsm_status tv_prox_slices(const TvSlices &s, float *pbuf, size_t pbuf_floats, 
     int dev = 0, sms = 0;
     cslsm_status e = device_info(dev, sms);
     if (e) return e;
-    if (s.theta > 0.f && s.T >= 1 && tv_get_mode() <= 1) {
+    if (s.theta > 0.f && s.T >= 1 && tv_get_mode() <= 1 && s.nslices <= kPhaseMaxSlices) {
         const PhaseShape f = phase_best(s.H, s.W, s.T, s.nslices, sms);
         const size_t need = f.P > 1 ? 4ull * s.nslices * s.H * s.W : 0;
         if (f.rpw && need <= pbuf_floats) return run_phases(s, f, pbuf, st);

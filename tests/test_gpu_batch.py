@@ -318,3 +318,26 @@ def test_batch_with_unaligned_caller_buffers(cs, shift):
         torch.cuda.synchronize()
         assert torch.equal(v, ref)
     batch.close()
+
+
+@pytest.mark.parametrize("T", [3, 20])
+def test_more_slices_than_a_grid_has_rows(cs, T):
+    """3,000 shots of 32 planes (Z = 96,000, gamma = 0): one solve gives the bits of the shots
+    solved by themselves."""
+    import torch
+
+    cs.set_tv_route(0)
+    H = W = 8
+    N, R = 3000, 32
+    g = torch.Generator().manual_seed(8)
+    masks = (torch.rand(N * R, H, W, generator=g) < 0.5).to(torch.uint8).cuda()
+    b = (torch.rand(N, H, W, generator=g) * R / 2).cuda()
+    prm = cs.Params(rho=1.0, lam=0.05, iters=3, denoiser="tv", tv_inner=T)
+    plan = cs.Plan(H, W, N, R, masks)
+    v = plan.solve(b, prm).cpu()
+    plan.close()
+    for n0 in (0, N - 5):
+        part = cs.Plan(H, W, 5, R, masks[n0 * R:(n0 + 5) * R].contiguous())
+        assert torch.equal(part.solve(b[n0:n0 + 5].contiguous(), prm).cpu(),
+                           v[n0 * R:(n0 + 5) * R])
+        part.close()
