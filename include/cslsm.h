@@ -175,9 +175,25 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
  *             by params->tv_inner Chambolle steps from p = 0;
  *   BM3D:     out = BM3D(in) at noise level params->bm3d_sigma (stage 1 then
  *             stage 2, see cslsm_bm3d_stage; scratch from cudaMallocAsync).
- * in, out: device [Z][H][W]; they must not overlap (neighbour reads). */
+ * in, out: device [Z][H][W]; they must not overlap (neighbour reads).
+ * TV allocates nothing for tv_inner <= 24 and takes 16 bytes a voxel from
+ * cudaMallocAsync beyond; with a workspace (cslsm_denoise_ws) it runs in launches of a
+ * few steps each, up to twice as fast, with the same bits. */
 cslsm_status cslsm_denoise(int denoiser, const float *in, float *out, int Z, int H, int W,
                            const cslsm_admm_params *params, void *stream);
+
+/* cslsm_denoise with device scratch of the caller's: ws, 16-byte aligned, ws_bytes long,
+ * free for other use once the work enqueued on `stream` is done; it must not overlap in
+ * or out.  A smaller one (or NULL) is accepted: the call then does as cslsm_denoise. */
+cslsm_status cslsm_denoise_ws(int denoiser, const float *in, float *out, int Z, int H, int W,
+                              const cslsm_admm_params *params, void *ws, size_t ws_bytes,
+                              void *stream);
+
+/* The scratch that makes cslsm_denoise_ws fastest on the current device: TV 16 bytes a
+ * voxel, or 0 where it needs none (few steps, more than 1 GB); 0 for the other
+ * denoisers and for arguments that cslsm_denoise_ws refuses. */
+size_t cslsm_denoise_workspace_bytes(int denoiser, int Z, int H, int W,
+                                     const cslsm_admm_params *params);
 
 /* ---- BM3D stages (the u-step denoiser of Sec. III-B / IV-C, by stage) ------
  * The variant built here, applied to each 2-D slice: 8 x 8 patches, reference

@@ -111,6 +111,7 @@ def lib() -> ctypes.CDLL:
         "cslsm_admm_solve": [P, P, ctypes.POINTER(AdmmParams), P, P, P,
                              ctypes.POINTER(AdmmStats), P],
         "cslsm_denoise": [I, P, P, I, I, I, ctypes.POINTER(AdmmParams), P],
+        "cslsm_denoise_ws": [I, P, P, I, I, I, ctypes.POINTER(AdmmParams), P, ctypes.c_size_t, P],
         "cslsm_psnr": [P, P, ctypes.c_size_t, P, P],
         "cslsm_ssim3d": [P, P, I, I, I, P, P],
         "cslsm_bm3d_match": [P, I, I, I, I, P, P, P],
@@ -121,6 +122,8 @@ def lib() -> ctypes.CDLL:
         fn = getattr(L, name)
         fn.argtypes = args
         fn.restype = I
+    L.cslsm_denoise_workspace_bytes.argtypes = [I, I, I, I, ctypes.POINTER(AdmmParams)]
+    L.cslsm_denoise_workspace_bytes.restype = ctypes.c_size_t
     L.cslsm_status_string.argtypes = [I]
     L.cslsm_status_string.restype = ctypes.c_char_p
     L.cslsm_last_error.argtypes = []
@@ -282,16 +285,34 @@ class Plan:
 
 
 def denoise(x: torch.Tensor, params: Params, out: torch.Tensor | None = None, stream=None):
-    """The u-step prior alone on each slice of x [Z,H,W] (cslsm_denoise)."""
+    """The u-step prior alone on each slice of x [Z,H,W] (cslsm_denoise_ws).  Large TV
+    calls take 16 bytes a voxel of scratch from torch's allocator; without the memory
+    they run slower."""
     if x.dim() == 2:
         x = x[None]
     Z, H, W = x.shape
     if out is None:
         out = torch.empty_like(x)
     cp = params.to_c()
-    _check(lib().cslsm_denoise(cp.denoiser, _dev(x, "x", torch.float32),
-                               _dev(out, "out", torch.float32, (Z, H, W)), Z, H, W,
-                               ctypes.byref(cp), _stream(stream)), "cslsm_denoise")
+    xp, op = _dev(x, "x", torch.float32), _dev(out, "out", torch.float32, (Z, H, W))
+    ref, L, ws, nbytes = ctypes.byref(cp), lib(), None, 0
+    # Scratch where the prox gains more than its allocation costs on the host (about 10 us):
+    # us a call without / with it 64 x 64, 20 steps 21 / 28; 512 x 512, 10 steps 19 / 28, 20
+    # steps 31 / 29; 16 x 512 x 512, 10 steps 110 / 79, 20 steps 315 / 156.
+    if cp.denoiser == TV and Z * H * W * cp.tv_inner >= 4 << 20:
+        nbytes = L.cslsm_denoise_workspace_bytes(cp.denoiser, Z, H, W, ref)
+    if nbytes:
+        try:
+            if stream is None:
+                ws = x.new_empty(nbytes // 4)
+            else:  # the scratch belongs to the stream that uses it
+                with torch.cuda.stream(stream):
+                    ws = x.new_empty(nbytes // 4)
+        except torch.cuda.OutOfMemoryError:
+            nbytes = 0
+    _check(L.cslsm_denoise_ws(cp.denoiser, xp, op, Z, H, W, ref,
+                              None if ws is None else ws.data_ptr(), nbytes, _stream(stream)),
+           "cslsm_denoise")
     return out
 
 

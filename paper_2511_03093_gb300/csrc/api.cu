@@ -615,12 +615,30 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
 cslsm_status cslsm_denoise(int denoiser, const float *in, float *out, int Z, int H, int W,
                            const cslsm_admm_params *prm, void *stream)
 {
+    return cslsm_denoise_ws(denoiser, in, out, Z, H, W, prm, nullptr, 0, stream);
+}
+
+size_t cslsm_denoise_workspace_bytes(int denoiser, int Z, int H, int W,
+                                     const cslsm_admm_params *prm)
+{
+    if (Z < 1 || H < 1 || W < 1 || (long long)Z * H * W >= (1ll << 31)) return 0;
+    if (check_params(prm, true) || denoiser != prm->denoiser || denoiser != CSLSM_DEN_TV ||
+        !(prm->lambda / prm->rho > 0.f))
+        return 0;
+    return sizeof(float) * tv_pbuf_floats(H, W, prm->tv_inner, Z);
+}
+
+cslsm_status cslsm_denoise_ws(int denoiser, const float *in, float *out, int Z, int H, int W,
+                              const cslsm_admm_params *prm, void *wsp, size_t ws_bytes,
+                              void *stream)
+{
     CHECK_ARG(in != nullptr && out != nullptr, "in and out must be non-NULL");
     CHECK_ARG(Z >= 1 && H >= 1 && W >= 1, "Z, H, W must be >= 1");
     CHECK_ARG((long long)Z * H * W < (1ll << 31), "Z*H*W must be < 2^31");
     cslsm_status st = check_params(prm, true);
     if (st) return st;
     CHECK_ARG(denoiser == prm->denoiser, "denoiser argument and params->denoiser differ");
+    CHECK_ARG((uintptr_t)wsp % 16 == 0, "the workspace must be 16-byte aligned");
     const size_t nv = (size_t)Z * H * W;
     if (denoiser != CSLSM_DEN_TIKHONOV) {
         const char *a = (const char *)in, *o = (const char *)out;
@@ -673,22 +691,16 @@ cslsm_status cslsm_denoise(int denoiser, const float *in, float *out, int Z, int
     a.theta = prm->lambda / prm->rho;
     a.tau = prm->tv_tau;
     a.T = prm->tv_inner;
+    // The phases' exchange comes from the caller: memory allocated and given back by each
+    // call is mapped anew after every synchronisation (200 us for one 256 x 256 slice, 1.2
+    // ms for 1024 x 1024 x 32, against 20 us and 2.5 ms for the whole prox in one launch).
+    const size_t need = a.theta > 0.f ? tv_pbuf_floats(H, W, a.T, Z) : 0;
+    if (a.T <= tv_max_steps_per_launch() || ws_bytes >= sizeof(float) * need)
+        return tv_prox_slices(a, (float *)wsp, wsp ? ws_bytes / sizeof(float) : 0, s);
     float *pbuf = nullptr;
-    size_t need = a.theta > 0.f ? tv_pbuf_floats(H, W, a.T, Z) : 0;
-    if (need && a.T <= tv_max_steps_per_launch()) {  // wanted, not needed
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CSLSM_CUDA(cudaStreamIsCapturing(s, &cap));
-        if (cap != cudaStreamCaptureStatusNone ||
-            cudaMallocAsync(&pbuf, sizeof(float) * need, s) != cudaSuccess) {
-            cudaGetLastError();
-            pbuf = nullptr;
-            need = 0;
-        }
-    } else if (need) {
-        CSLSM_CUDA(cudaMallocAsync(&pbuf, sizeof(float) * need, s));
-    }
+    CSLSM_CUDA(cudaMallocAsync(&pbuf, sizeof(float) * need, s));
     st = tv_prox_slices(a, pbuf, need, s);
-    if (pbuf) cudaFreeAsync(pbuf, s);
+    cudaFreeAsync(pbuf, s);
     return st;
 }
 
