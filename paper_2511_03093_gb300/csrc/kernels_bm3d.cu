@@ -90,9 +90,13 @@ __global__ void bm3d_prep_kernel(const S *__restrict__ src, const S *__restrict_
 // middle rows; each of the 8 lanes of a reference keeps the 6 least of its pairs of
 // adjacent candidates, and the 16th smallest of those 48 SSDs bounds the 16th
 // smallest of the window (the reference itself is one).  Pass 2 forms the products
-// of the whole window and keeps the keys up to the bound (about 40), in lists of its
+// of the whole window and keeps the keys up to the bound (about 40 of a noisy one), in lists of its
 // own per lane and reference; a list that fills up drops all but its 16 smallest and
 // lowers its bound.  The lanes of a reference then sort and merge their lists.
+// Where many candidates tie (a dark background, saturation), a cut list also bounds the
+// position: rows below that of its last key need a smaller SSD.  Without that every
+// tied candidate was appended (4 x 512 x 512 of one value: 1,421 us a launch; one warp
+// per reference on dp4a 622; now 423).
 //   kSplit warps share a block of references, each with every kSplit-th tile column:
 // two on CTAs of 2 x 2 blocks, which share the staging, or six on CTAs of one block
 // where the larger CTAs would leave a quarter of the SMs idle.  Both in us a launch:
@@ -178,17 +182,20 @@ __device__ __forceinline__ void merge16(uint32_t (&k)[16], F other)
     for (int i = 0; i < 16; ++i) k[i] = q[i];
 }
 
-// A lane's full list down to its 16 smallest keys; returns the largest of them.
+// A lane's list of n keys (16 < n <= kMCap) down to its 16 smallest; returns the largest
+// of them.
 __device__ __noinline__ uint32_t shrink_list(uint32_t *list, int n)
 {
-    uint32_t k[16];
+    static_assert(kMCap == 32, "two sorted halves");
+    uint32_t k[16], q[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) k[i] = kMNone;
-    for (int j = 0; j < n; ++j) {
-        uint32_t key = list[j * 32];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) order(k[i], key);
+    for (int i = 0; i < 16; ++i) {
+        k[i] = list[i * 32];
+        q[i] = 16 + i < n ? list[(16 + i) * 32] : kMNone;
     }
+    sort16(k);
+    sort16(q);
+    merge16(k, [&](int i) { return q[i]; });
 #pragma unroll
     for (int i = 0; i < 16; ++i) list[i * 32] = k[i];
     return k[15];
@@ -240,7 +247,8 @@ __device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *b
                                            MatchFetch &f, const float (&r0)[2],
                                            const float (&r1)[2], int y, uint32_t l,
                                            uint32_t (&R)[7], float (&best)[2][kMBest],
-                                           uint32_t *list, uint32_t (&at)[2], float (&vt)[2])
+                                           uint32_t *list, uint32_t (&at)[2], float (&vt)[2],
+                                           bool &tied, int (&lim)[2])
 {
     uint32_t w[11];
     float d[4][4];
@@ -263,6 +271,11 @@ __device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *b
                      w[i + 2 * k + 1]);
 #pragma unroll
     for (int i = 0; i < 7; ++i) R[i] = w[i + 4];
+    float t0 = vt[0], t1 = vt[1];
+    if (PASS == 2 && tied) {  // below the row of the last key kept, an equal SSD comes later
+        t0 = y > lim[0] ? t0 - 1.f : t0;
+        t1 = y > lim[1] ? t1 - 1.f : t1;
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const bool v0 = WHOLE || (unsigned)(y + i - m.ylo[0]) <= (unsigned)(m.yhi[0] - m.ylo[0]);
@@ -278,7 +291,7 @@ __device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *b
                 best[r][0] = fminf(best[r][0], v);
             }
         } else {
-            const float b0 = v0 ? vt[0] : 0.f, b1 = v1 ? vt[1] : 0.f;
+            const float b0 = v0 ? t0 : 0.f, b1 = v1 ? t1 : 0.f;
             const uint32_t li = l + (uint32_t)(i * 128);
             append_if(at[0], (__float_as_uint(d[i][0]) << 13) + li, d[i][0], b0);
             append_if(at[1], (__float_as_uint(d[i][2]) << 13) + li, d[i][2], b1);
@@ -294,12 +307,15 @@ __device__ __forceinline__ void match_rows(const MatchLane &m, const uint32_t *b
                 const uint32_t top = shrink_list(list, (int)(at[0] - l0) / 128);
                 at[0] = l0 + 16 * 128;
                 vt[0] = fminf(vt[0], kMBias + (float)(top >> 13));
+                lim[0] = (int)((top >> 7) & 63u) - m.ly;
             }
             if (at[1] > l1 + kMFull * 128) {
                 const uint32_t top = shrink_list(list + kMCap * 32, (int)(at[1] - l1) / 128);
                 at[1] = l1 + 16 * 128;
                 vt[1] = fminf(vt[1], kMBias + (float)(top >> 13));
+                lim[1] = (int)((top >> 7) & 63u) - m.ly;
             }
+            tied = true;
             __syncwarp();
         }
     }
@@ -313,6 +329,8 @@ __device__ __forceinline__ void match_scan(const MatchLane &m, int c0, int first
                                            uint32_t (&at)[2], float (&vt)[2])
 {
     constexpr float kPen = 16777216.f;
+    bool tied = false;  // a list has been cut (the same in every lane)
+    int lim[2] = {kMSpan, kMSpan};  // the window row of the last key it kept
     for (int c = c0; c < kMSpan / 8; c += SPLIT) {
         const int x = m.lx + 8 * c + 2 * m.t;
         const bool v0 = x >= m.xlo && x <= m.xhi, v1 = x + 1 >= m.xlo && x + 1 <= m.xhi;
@@ -336,9 +354,11 @@ __device__ __forceinline__ void match_scan(const MatchLane &m, int c0, int first
                 sp += 4 * CAND;
             }
             if (y >= m.all_lo && y + 3 <= m.all_hi)
-                match_rows<PASS, true, CAND>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
+                match_rows<PASS, true, CAND>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt,
+                                              tied, lim);
             else
-                match_rows<PASS, false, CAND>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt);
+                match_rows<PASS, false, CAND>(m, bp, sp, f, r0, r1, y, l, R, best, list, at, vt,
+                                               tied, lim);
             l += 4 * 128;
         }
     }

@@ -96,6 +96,35 @@ def test_match_lists_on_ties_and_edges(cs, H, W, stage):
         np.testing.assert_array_equal(lists[z], idx)
 
 
+def _tied(H, W):
+    """Windows of one value, whole or in part: every candidate ties."""
+    y, x = np.mgrid[:H, :W]
+    noise = np.random.default_rng(H + W).random((H, W))
+    yield np.full((H, W), 0.25)
+    yield np.where(y > H // 2, noise, 0.0)         # dark above, noisy below
+    yield np.where(x > W // 2, noise, 1.0)         # saturated on the left
+    yield np.where((x // 5 + y // 7) % 2, 0.0, 0.6)  # squares
+    yield (y % 3 < 1).astype(float)                # rows
+
+
+# 1 copy: six warps to a block of references; as many as it takes: two warps
+@pytest.mark.parametrize("few", [True, False])
+@pytest.mark.parametrize("H,W", [(8, 9), (21, 33), (47, 48), (64, 35), (75, 90)])
+@pytest.mark.parametrize("stage", [1, 2])
+def test_match_lists_where_all_candidates_tie(cs, H, W, stage, few):
+    base = np.stack([*_patterns(H, W), *_tied(H, W)]).astype(np.float32)
+    ctas = -(-cs.lib().cslsm_bm3d_num_refs(H, 8) // 8) * -(-cs.lib().cslsm_bm3d_num_refs(8, W) // 8)
+    copies = 1 if few else -(-152 // (ctas * len(base)))
+    lists, counts = cs.bm3d_match(to_dev(np.concatenate([base] * copies)), stage)
+    lists = lists.cpu().numpy().reshape(copies, len(base), -1, 16)
+    counts = counts.cpu().numpy().reshape(copies, len(base), -1)
+    for z in range(len(base)):
+        idx, cnt = oracle.bm3d_match(base[z], stage)
+        for c in range(copies):
+            np.testing.assert_array_equal(counts[c, z], cnt)
+            np.testing.assert_array_equal(lists[c, z], idx)
+
+
 def test_match_ties_on_constant_image(cs):
     img = np.full((1, 40, 44), 0.25, dtype=np.float32)
     lists, counts = cs.bm3d_match(to_dev(img), 1)
