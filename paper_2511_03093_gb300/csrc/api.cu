@@ -433,7 +433,7 @@ cslsm_status cslsm_admm_solve(cslsm_plan plan, const float *b, const cslsm_admm_
         cudaGetLastError();  // the failed allocation's (non-sticky) error
     }
     if (prm->denoiser == CSLSM_DEN_TIKHONOV && !use_tol && prm->iters >= 1 &&
-        tikhonov_solve_applies(g)) {
+        tikhonov_solve_applies(g, store, prm->init_user != 0, gam, prm->iters)) {
         st = launch_tikhonov_solve(g, masks_of(plan), store, u_io, d_io, prm->init_user != 0, b,
                                    prm->rho, prm->lambda, gam, prm->iters, v_out, s);
         if (st) return st;

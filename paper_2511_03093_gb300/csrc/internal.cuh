@@ -82,14 +82,15 @@ cslsm_status launch_xupdate_w(const Geom &g, Masks m, int storage, const void *u
                               double *partials, int nblocks_red, cudaStream_t s,
                               const int *stop = nullptr);
 
-// One whole ADMM iteration with the Tikhonov prior fused into one pass:
-// v-update, Gauss-Seidel Tikhonov sweep along z (gamma > 0) and dual update.
 // The whole Tikhonov solve of one shot in one launch (fixed iteration count >= 1): from
-// u, d if `init`, else from zeros; u^K, d^K to u, d unless null.
-bool tikhonov_solve_applies(const Geom &g);
+// u, d if `init`, else from zeros; u^K, d^K to u, d unless null.  Where it is the faster
+// way:
+bool tikhonov_solve_applies(const Geom &g, int storage, bool init, float gam, int iters);
 cslsm_status launch_tikhonov_solve(const Geom &g, Masks m, int storage, void *u, void *d,
                                    bool init, const float *b, float rho, float lam, float gam,
                                    int iters, float *v_out, cudaStream_t s);
+// One whole ADMM iteration with the Tikhonov prior fused into one pass:
+// v-update, Gauss-Seidel Tikhonov sweep along z (gamma > 0) and dual update.
 cslsm_status launch_tikhonov_iter(const Geom &g, Masks m, int storage, void *u, void *d,
                                   const float *b, float rho, float lam, float gam, float *v_out,
                                   float *vprev, double *partials, int nblocks_red, cudaStream_t s,

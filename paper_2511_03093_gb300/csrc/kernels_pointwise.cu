@@ -648,7 +648,31 @@ cslsm_status tikhonov_solve_typed(const Geom &g, Masks m, void *u, void *d, bool
     return CSLSM_OK;
 }
 
-bool tikhonov_solve_applies(const Geom &g) { return g.N == 1 && g.R <= CSLSM_MAX_R; }
+// Few iterations from a given state are bound by moving that state, which
+// tikhonov_iter_kernel does in wider accesses than one thread a pixel column; with plane
+// counts that no instantiation matches exactly it is the faster one up to `few` iterations
+// (otherwise for one iteration of 16-bit state with gamma = 0: BF16 16 planes 51 / 57, 32
+// planes 119 / 131, at 512 x 512 38 / 32).
+// us, one launch an iteration / one launch, 1024 x 1024: FP32 20 planes, 1 iteration 91 /
+// 103 (12 planes 54 / 53); BF16 20 planes 1: 75 / 114, 2: 135 / 151, 3: 197 / 192 (512 x
+// 512, 2: 31 / 30); FP16 20 planes 1: 57 / 113, 2: 96 / 129, 3: 130 / 146, 4: 170 / 165, 12
+// planes 2: 53 / 57, 3: 73 / 64.  From zeros one launch is always the faster.
+bool tikhonov_solve_applies(const Geom &g, int storage, bool init, float gam, int iters)
+{
+    if (g.N != 1 || g.R > CSLSM_MAX_R) return false;
+    const int Z = g.Z();
+    const long long nv = g.voxels();
+    if (!init || g.HW() < 1 << 18) return true;
+    int few;
+    if (Z == 8 || Z == 16 || Z == 32)
+        few = gam == 0.f && (storage == CSLSM_STORE_BF16   ? Z < 32 || nv > 1 << 23
+                             : storage == CSLSM_STORE_FP16 ? Z < 32
+                                                           : false);
+    else if (storage == CSLSM_STORE_FP32) few = Z > 16;
+    else if (storage == CSLSM_STORE_BF16) few = nv >= 1 << 23 ? 2 : 1;
+    else few = nv <= 1 << 22 ? 1 : nv >= 1 << 23 && Z > 16 ? 3 : 2;
+    return iters > few;
+}
 
 cslsm_status launch_tikhonov_solve(const Geom &g, Masks m, int storage, void *u, void *d,
                                    bool init, const float *b, float rho, float lam, float gam,

@@ -100,3 +100,26 @@ def test_one_launch_tikhonov_equals_iteration_launches(cs, Z, gamma, storage):
             assert torch.equal(x, y)
     assert torch.equal(out[2][0], out[0][0])
     plan.close()
+
+
+# either side of each line of the choice: few iterations from a given state, by type and size
+@pytest.mark.parametrize("storage,Z,H,iters", [("fp32", 20, 512, 1), ("fp32", 20, 511, 1),
+                                               ("bf16", 8, 520, 1), ("bf16", 20, 648, 2),
+                                               ("bf16", 20, 648, 3), ("fp16", 12, 600, 2),
+                                               ("fp16", 20, 648, 3), ("fp16", 20, 648, 4)])
+@pytest.mark.parametrize("gamma", [0.0, 0.2])
+def test_few_tikhonov_iterations_from_a_state(cs, storage, Z, H, iters, gamma):
+    g = torch.Generator().manual_seed(Z + H)
+    masks = (torch.rand(Z, H, H, generator=g) < 0.5).to(torch.uint8).cuda()
+    b = torch.rand(1, H, H, generator=g).cuda()
+    u0, d0 = (torch.rand(Z, H, H, generator=g).to(cs.STORAGE_DTYPE[storage]) for _ in range(2))
+    plan = cs.Plan(H, H, 1, Z, masks)
+    out = []
+    for tol in (0.0, 1e-30):  # a tolerance that is never met: one launch an iteration
+        prm = cs.Params(rho=0.9, lam=0.05, gamma=gamma, iters=iters, denoiser="tikhonov", tol=tol,
+                        check_every=100, storage=storage)
+        u, d = u0.cuda(), d0.cuda()
+        out.append((plan.solve(b, prm, u=u, d=d, init_user=True), u, d))
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
+    plan.close()
