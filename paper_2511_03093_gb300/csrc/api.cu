@@ -824,20 +824,28 @@ cslsm_status cslsm_batch_create(cslsm_batch *out, const cslsm_batch_item *items,
     // steps per phase: by rule unless a phase length is set or timing a few
     // candidates on the batch itself is asked for (autotune mode 1).  At most 10
     // steps, or balanced phases of at most 8 (T = 20: 7) where a level of the items
-    // fills the grid: fewer steps waste less on halos, more phases cost loads and,
-    // with few tiles in flight, waits.  ms at 10 / 7 steps, by tiles of a level over
-    // CTAs: 12 items BF16 (3.5) 58.7 / 53.1; 1 x 1024 x 1024 x 32 gamma = 0 (22) 14.9 /
-    // 13.6; 700 x 333 x 20 (3.07) 2.80 / 2.88; 512 x 512 x 16 (2.7) 1.99 / 2.09; 4
-    // items (0.9) 35.2 / 36.5.
+    // fills the grid (with few tiles in flight more phases cost waits) and the work is
+    // less: a unit costs about 4 steps besides its own, so tiles x (4 phases + T).
+    // Fewer steps make larger tiles, which a slice's size turns into fewer of them or
+    // not.  ms at 10 steps / balanced: 12 items BF16, T = 20 58.7 / 53.1; 1 x 1024 x 1024 x
+    // 32 gamma = 0, T = 20 14.9 / 13.6, T = 40 27.6 / 26.3; 10 x 512 x 512 x 16 gamma = 0, T
+    // = 20 5.8 / 5.4 and T = 40 10.6 / 11.2; 12 x 253 x 317 x 8, T = 20 1.29 / 1.40; few tiles:
+    // 700 x 333 x 20 2.80 / 2.88, 4 items 35.2 / 36.5.  Over 7 sets of items, 13 T from 11 to
+    // 80, gamma = 0 and 0.2, BF16 and FP32 the choice is 3 % behind 10 steps at most.
     int kbest = std::min(std::max(T, 1), 10);
     if (T > 10) {
         const int phases = (T + 7) / 8, kbal = (T + phases - 1) / phases;
         long long tiles = 0;
+        double wbal = 0.0, w10 = 0.0;
         for (const BatchItemSpec &it : spec.items) {
             const int Z = it.N * it.R;
-            tiles += batch_tiles_per_slice(it.H, it.W, kbal) * (prm->gamma > 0.f && Z > 1 ? 1 : Z);
+            const long long t = batch_tiles_per_slice(it.H, it.W, kbal);
+            tiles += t * (prm->gamma > 0.f && Z > 1 ? 1 : Z);
+            wbal += (double)Z * t * (4.0 * phases + T);
+            w10 += (double)Z * batch_tiles_per_slice(it.H, it.W, kbest) *
+                   (4.0 * ((T + kbest - 1) / kbest) + T);
         }
-        if (3 * tiles >= 10 * 3ll * sms) kbest = kbal;  // three CTAs per SM
+        if (3 * tiles >= 10 * 3ll * sms && wbal < 0.96 * w10) kbest = kbal;  // three CTAs per SM
     }
     const int kset = g_batch_k;
     if (kset > 0) {

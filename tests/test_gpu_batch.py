@@ -341,3 +341,26 @@ def test_more_slices_than_a_grid_has_rows(cs, T):
         assert torch.equal(part.solve(b[n0:n0 + 5].contiguous(), prm).cpu(),
                            v[n0 * R:(n0 + 5) * R])
         part.close()
+
+
+# balanced phases where they are less work: the larger tiles of fewer steps save tiles at
+# 512 x 512, not at 253 x 317; at T = 40 they cost a phase more; few tiles keep 10 steps
+@pytest.mark.parametrize("shapes,T,k", [([(16, 512, 512)] * 10, 20, 7),
+                                        ([(16, 512, 512)] * 10, 40, 10),
+                                        ([(8, 253, 317)] * 12, 20, 10),
+                                        ([(8, 253, 317)] * 12, 12, 6),
+                                        ([(4, 96, 80)], 20, 10)])
+def test_steps_per_phase(cs, shapes, T, k):
+    import torch
+
+    items = []
+    for Z, H, W in shapes:
+        masks = torch.ones(Z, H, W, dtype=torch.uint8, device="cuda")
+        items.append((cs.Plan(H, W, 1, Z, masks), torch.ones(1, H, W, device="cuda"),
+                      torch.empty(Z, H, W, device="cuda")))
+    bt = cs.Batch(items, cs.Params(rho=1.0, lam=0.05, iters=1, denoiser="tv", tv_inner=T,
+                                   storage="bf16"))
+    assert bt.info()["steps_per_phase"] == k
+    bt.close()
+    for p, _, _ in items:
+        p.close()
