@@ -278,7 +278,7 @@ cslsm_status cslsm_batch_create(cslsm_batch *batch, const cslsm_batch_item *item
  *   mode 0 (default): the per-launch path, which runs the prox as a few launches
  *          of several steps each (their exchange of the dual field, 16 bytes a
  *          voxel up to 1 GB, belongs to the plan); the batch with BF16 state,
- *          or beyond that size, when one phase level holds at least 4 tiles per
+ *          FP16 state of large volumes, or beyond that size, when one phase level holds at least 4 tiles per
  *          SM (large volumes); a batch that does not fit in device memory
  *          leaves the solve to the per-launch path, and so does stream capture;
  *   mode 1: always the per-launch path;   mode 2: always the batch (a capture

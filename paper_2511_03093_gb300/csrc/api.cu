@@ -312,9 +312,17 @@ bool tv_route_applies(const cslsm_plan_s *plan, const cslsm_admm_params *prm, fl
         prm->init_user || u_io != nullptr || prm->iters < 1)
         return false;
     if (mode == 2) return true;
-    // the phase launches are faster but with BF16 state (1024 x 1024 x 32: 1,413 us an
-    // iteration here, 1,541 there; FP32 1,350 / 1,221, FP16 512 x 512 x 16 194 / 185)
-    if (phases && prm->storage != CSLSM_STORE_BF16 && tv_get_mode() <= 1 &&
+    // The phase launches are faster but with BF16 state (1024 x 1024 x 32: 1,413 us an
+    // iteration here, 1,541 there; FP32 1,350 / 1,221), and FP16 state of large volumes
+    // where the batch updates x in wide accesses.  FP16, us an iteration here / there:
+    // 1024 x 1024 x 32, 20 steps 1,301 / 1,487, 5 steps 453 / 484; 2048 x 2048 x 8, 20 1,257 /
+    // 1,422, 5 432 / 420; 768 x 768 x 32, 20 776 / 830, 5 266 / 275; 16 planes of it, 20 403 /
+    // 401, 5 137 / 116; 999 x 701 x 24, 20 903 / 760.
+    const long long nv = plan->g.voxels();
+    const bool wide_fp16 = prm->storage == CSLSM_STORE_FP16 && plan->g.HW() % 4 == 0 &&
+                           (prm->tv_inner >= 15 ? nv >= 1 << 24
+                                                : nv >= 1 << 25 && plan->g.R >= 32);
+    if (phases && prm->storage != CSLSM_STORE_BF16 && !wide_fp16 && tv_get_mode() <= 1 &&
         tv_phases_fit(plan->g.H, plan->g.W, plan->g.Z()))
         return false;
     int dev = 0, sms = 0;

@@ -364,3 +364,24 @@ def test_steps_per_phase(cs, shapes, T, k):
     bt.close()
     for p, _, _ in items:
         p.close()
+
+
+# FP16 state: the batch (one launch) for large volumes whose x-update it does in wide
+# accesses, launches of a few steps otherwise
+@pytest.mark.parametrize("Z,H,W,T,batch", [(32, 1024, 1024, 3, True), (16, 1024, 1024, 15, True),
+                                           (16, 1024, 1024, 3, False), (16, 1024, 1023, 15, False),
+                                           (32, 1021, 1027, 20, False)])
+def test_fp16_route(cs, Z, H, W, T, batch):
+    import torch
+
+    cs.set_tv_route(0)
+    masks = torch.ones(Z, H, W, dtype=torch.uint8, device="cuda")
+    b = torch.rand(1, H, W, device="cuda") * Z
+    plan = cs.Plan(H, W, 1, Z, masks)
+    prm = cs.Params(rho=1.0, lam=0.05, iters=2, denoiser="tv", tv_inner=T, storage="fp16")
+    n0 = cs.launch_count()
+    v = plan.solve(b, prm)
+    assert (cs.launch_count() - n0 <= 2) == batch
+    cs.set_tv_route(1)
+    assert torch.equal(plan.solve(b, prm), v)
+    plan.close()
