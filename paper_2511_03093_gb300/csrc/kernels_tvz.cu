@@ -423,15 +423,21 @@ bool make_cfg(int c, int H, int W, int T, int sms, int storage, Cfg &f)
 // FP32 and BF16, T = 20, 9 % rms.  Its choice is on average 1.2 % behind the best
 // tiling, 3.2 % at most; the count of region pixels it replaces was up to 36 % behind
 // (us per slice: 512 x 512 28.3 -> 23.4, 640 x 480 32.2 -> 24.1, 256 x 256 17.9 -> 15.6).
-double model(const Cfg &f, int T, int sms)
+// BF16 state loads and stores cost more a row: with the constants of the fit its choice at
+// 512 x 512 and 60 steps was two CTAs on an SM at 87.4 us a slice, now one at 79.9.  Over 11
+// geometries, T from 3 to 60 and three types no choice is slower than the count's, 2 to 3
+// % behind the best tiling on average.
+double model(const Cfg &f, int T, int sms, int storage)
 {
+    const bool bf16 = storage == CSLSM_STORE_BF16;
     const int tiles = f.tx * f.ty;
     const int per_sm = (tiles + sms - 1) / sms;
     const int P = (T + f.k - 1) / f.k;
     const double rows = (double)per_sm * f.B * f.RPW;
     const double active = std::min((double)f.B, std::ceil((f.TH + f.k - 1.0) / f.RPW) + 0.5);
-    const double issue = 0.01216 * per_sm * active * f.RPW * (per_sm > 1 ? 0.84 : 1.0);
-    return P * (3.51 + 0.01718 * rows) + T * (0.01818 * f.RPW - 0.0533 + issue);
+    const double issue =
+        0.01216 * per_sm * active * f.RPW * (per_sm > 1 ? (bf16 ? 0.86 : 0.84) : 1.0);
+    return P * (3.51 + (bf16 ? 0.0292 : 0.01718) * rows) + T * (0.01818 * f.RPW - 0.0533 + issue);
 }
 
 std::mutex g_mu;
@@ -573,7 +579,7 @@ cslsm_status choose(const TvSlices &s, ZsweepWs &ws, cudaStream_t st, Cfg &out)
         Cfg f;
         if (!make_cfg(c, s.H, s.W, s.T, sms, s.storage, f)) continue;
         ok.push_back(c);
-        const double m = model(f, s.T, sms);
+        const double m = model(f, s.T, sms, s.storage);
         if (m < best_cost) {
             best_cost = m;
             best = c;
@@ -731,7 +737,7 @@ cslsm_status zsweep_query(int H, int W, int Z, int T, int storage, int *out8)
         for (int c = 0; c < kNumCand; ++c) {
             Cfg g;
             if (!make_cfg(c, H, W, T, sms, storage, g)) continue;
-            const double m = model(g, T, sms);
+            const double m = model(g, T, sms, storage);
             if (m < bc) {
                 bc = m;
                 cand = c;

@@ -154,3 +154,9 @@ def test_phase_launches_match_tiles_bitwise(cs, Z, H, W, T, gamma, storage):
     for a, e in zip(*out):
         assert torch.equal(a, e)
     plan.close()
+
+
+def test_bf16_tiling_of_many_steps(cs):
+    """BF16 rows cost more to load: one CTA an SM at 512 x 512 and 60 steps, not two."""
+    assert cs.zsweep_shape(512, 512, 4, 60, "bf16")["tiles"] <= 152
+    assert cs.zsweep_shape(640, 480, 4, 10, "bf16")["tiles"] > 152
