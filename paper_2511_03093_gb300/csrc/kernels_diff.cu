@@ -59,6 +59,35 @@ struct Pair32 {
         lo += ((hi - (s - v)) + (h - v)) + l;
         hi = s;
     }
+    // adds (h + l) x f, f = (f.x + f.y), products of the leading parts exact
+    __device__ __forceinline__ void add_scaled(float h, float l, float2 f)
+    {
+        const float p = h * f.x;
+        add(p, fmaf(h, f.x, -p) + fmaf(l, f.x, h * f.y));
+    }
+};
+
+// Two such sums side by side, of a lane's two columns.
+struct Pairs32 {
+    float2 hi, lo;
+    __device__ __forceinline__ void add(float2 h, float2 l)
+    {
+        const float2 s = add2(hi, h), v = sub2(s, hi);
+        lo = add2(lo, add2(add2(sub2(hi, sub2(s, v)), sub2(h, v)), l));
+        hi = s;
+    }
+    __device__ __forceinline__ void add(float2 h)
+    {
+        const float2 s = add2(hi, h), v = sub2(s, hi);
+        lo = add2(lo, add2(sub2(hi, sub2(s, v)), sub2(h, v)));
+        hi = s;
+    }
+    __device__ __forceinline__ Pair32 total() const
+    {
+        Pair32 t = {hi.x, lo.x};
+        t.add(hi.y, lo.y);
+        return t;
+    }
 };
 
 // Adds the block's sums of v[0 .. N) to acc[idx[.]][blockIdx.x % kAccCopies].
@@ -204,7 +233,8 @@ struct HuberArgs {
     float *Wbar, *Abar, *Cbar;  // reverse, last phase (Abar may be Cbar: Z = 2)
     double *acc;
     Geo g;
-    float rho, gam, theta, inv_theta, tau, kappa, eps;
+    float rho, gam, theta, inv_theta, tau, kappa;
+    float2 it2, kfac;  // 1 / theta^2 and tau eps / theta^2, each in two parts
     int t0, ns;  // steps t0 .. t0 + ns - 1 (reverse: downwards)
     int T;
     int hh, hc, TH, TW, tx;
@@ -659,7 +689,7 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
         for (int i = 0; i <= RPW; ++i)
             u[i] = ld_pair(ub, t.off(i, W), t.row_in(i) && t.in0, t.row_in(i) && t.in1, a.pair);
         proj(t.gi0 + t.r0 - 1, up1, up2);
-        float part = 0.f;
+        Pairs32 part = {};
 #pragma unroll
         for (int i = 0; i < RPW; ++i) {
             float2 x1, x2;
@@ -668,13 +698,13 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
             const float2 dv = add2(sub2(x1, up1), sub2(x2, make_float2(l, x2.x)));
             up1 = x1;
             if (t.row_own(i))
-                part -= (t.own0 ? u[i].x * dv.x : 0.f) + (t.own1 ? u[i].y * dv.y : 0.f);
+                part.add(make_float2(t.own0 ? -u[i].x * dv.x : 0.f, t.own1 ? -u[i].y * dv.y : 0.f));
             const float ur = __shfl_down_sync(FULL, u[i].x, 1);
             b1[i] = mul2(sub2(u[i + 1], u[i]), splat(a.theta));
             b2[i] = mul2(sub2(make_float2(u[i].y, ur), u[i]), splat(a.theta));
             t.mask(i, b1[i], b2[i]);
         }
-        sum[0].hi = part;
+        sum[0] = part.total();
     }
 #pragma unroll
     for (int i = 0; i < RPW; ++i) sq[i] = make_float2(0.f, 0.f);
@@ -688,7 +718,7 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
     else huber_reverse<false, NW, RPW>(a, t, sb, ring, groups, b1, b2, sq, tk, tk_err);
     // hbar -= sum qbar / theta and the h / theta partial <qbar, h> / theta^2
     const float *ub = a.Ubar + bi * a.g.NV();
-    float tq = 0.f;
+    Pairs32 tqs = {};
     float2 h[RPW];
 #pragma unroll
     for (int i = 0; i < RPW; ++i) {
@@ -697,12 +727,14 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
         h[i] = ld_pair(Hb, o, o0, o1, a.pair);
         hb[i] = ld_pair(a.Pin ? Hbar : ub, o, o0, o1, a.pair);
         hb[i] = fma2(sq[i], splat(-a.inv_theta), hb[i]);
-        tq += (o0 ? sq[i].x * h[i].x : 0.f) + (o1 ? sq[i].y * h[i].y : 0.f);
+        const float2 q = make_float2(o0 ? sq[i].x : 0.f, o1 ? sq[i].y : 0.f);
+        const float2 qh = mul2(q, h[i]);
+        tqs.add(qh, fma2(q, h[i], mul2(qh, splat(-1.f))));
     }
+    const Pair32 tq = tqs.total();
     // kappa = eps / theta: d/dtheta of -tau kappa <abar, p>
-    const float it2 = a.inv_theta * a.inv_theta, kfac = a.tau * a.eps * it2;
-    sum[0].add(kfac * tk, kfac * tk_err);
-    sum[0].add(it2 * tq, 0.f);
+    sum[0].add_scaled(tk, tk_err, a.kfac);
+    sum[0].add_scaled(tq.hi, tq.lo, a.it2);
     if (a.Pout) {
         float *Q1 = a.Pout + (size_t)bi * 2 * HW, *Q2 = Q1 + HW;
 #pragma unroll
@@ -718,7 +750,7 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
         float *Wb = a.Wbar + bi * a.g.NV(), *Ab = a.Abar + bi * a.g.NV(),
               *Cb = a.Cbar + bi * a.g.NV();
         const float den = a.rho + 2.f * a.gam, cw = a.rho / den, cn = a.gam / den;
-        float rb = 0.f, gb = 0.f;
+        Pairs32 rb = {}, gb = {};
 #pragma unroll
         for (int i = 0; i < RPW; ++i) {
             const bool o0 = t.row_own(i) && t.own0, o1 = t.row_own(i) && t.own1;
@@ -731,14 +763,14 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
                         a.pair);
                 st_pair(Cb, o, fma2(splat(cn), hb[i], ld_pair(Cb, o, o0, o1, a.pair)), o0, o1,
                         a.pair);
-                gb += (o0 ? hb[i].x * (s.x - 2.f * h[i].x) / den : 0.f) +
-                      (o1 ? hb[i].y * (s.y - 2.f * h[i].y) / den : 0.f);
+                gb.add(make_float2(o0 ? hb[i].x * (s.x - 2.f * h[i].x) / den : 0.f,
+                                   o1 ? hb[i].y * (s.y - 2.f * h[i].y) / den : 0.f));
             }
-            rb += (o0 ? hb[i].x * (w.x - h[i].x) / den : 0.f) +
-                  (o1 ? hb[i].y * (w.y - h[i].y) / den : 0.f);
+            rb.add(make_float2(o0 ? hb[i].x * (w.x - h[i].x) / den : 0.f,
+                               o1 ? hb[i].y * (w.y - h[i].y) / den : 0.f));
         }
-        sum[1].hi = rb;
-        sum[2].hi = gb;
+        sum[1] = rb.total();
+        sum[2] = gb.total();
     }
     if (a.Pout) {
         Pair32 one[1] = {sum[0]};
@@ -924,7 +956,9 @@ HuberArgs huber_args(const Geo &g, const Prm &P, int k, bool pair)
     a.theta = P.theta();
     a.inv_theta = a.theta > 0.f ? 1.f / a.theta : 0.f;
     a.tau = P.tau;
-    a.eps = P.eps;
+    const double it2 = (double)a.inv_theta * a.inv_theta, kfac = it2 * P.tau * P.eps;
+    a.it2 = make_float2((float)it2, (float)(it2 - (float)it2));
+    a.kfac = make_float2((float)kfac, (float)(kfac - (float)kfac));
     a.kappa = a.theta > 0.f ? P.eps / a.theta : 0.f;
     a.T = P.steps();
     a.hh = k + 1;
