@@ -108,8 +108,9 @@ __device__ __forceinline__ void block_acc(Pair32 (&v)[N], double *acc, const int
         Pair32 t = s_part[threadIdx.x][0];
         for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
             t.add(s_part[threadIdx.x][w].hi, s_part[threadIdx.x][w].lo);
+        // an infinite sum has no second part
         atomicAdd(acc + idx[threadIdx.x] * kAccCopies + blockIdx.x % kAccCopies,
-                  (double)t.hi + (double)t.lo);
+                  isfinite(t.hi) ? (double)t.hi + (double)t.lo : (double)t.hi);
     }
 }
 

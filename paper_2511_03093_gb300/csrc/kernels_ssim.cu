@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kZThreads) ssim_z_kernel(const float *__restri
         }
     }
     __shared__ double sa[kZThreads];
-    sa[threadIdx.x] = (double)hi + (double)lo;
+    sa[threadIdx.x] = isfinite(hi) ? (double)hi + (double)lo : (double)hi;
     __syncthreads();
     for (int s = kZThreads / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s) sa[threadIdx.x] += sa[threadIdx.x + s];

@@ -106,6 +106,16 @@ def test_theta_that_underflows_leaves_the_prox_out(cs, Z, keep):
     assert float(l_.grad) == 0.0
 
 
+def test_an_overflowing_scalar_gradient_is_infinite(cs):
+    """Every pixel's share of dL/drho overflows to -infinity: so does the sum, not to NaN."""
+    logits, b, _ = _problem(51, 1, 1, 24, 20)
+    lg = logits.cuda().requires_grad_(True)
+    r, l_, gm = _scalars()
+    v = cs.unrolled_admm(lg, (100.0 + b).cuda(), r, l_, gm, **dict(CFG, iters=1))
+    v.backward(torch.full_like(v, 3e38))
+    assert float(r.grad) == -float("inf")
+
+
 def test_checkpoint_period_does_not_change_gradients(cs):
     logits, b, _ = _problem(5, 1, 4, 20, 18)
     vbar = torch.randn(1, 4, 20, 18, generator=torch.Generator().manual_seed(6)).cuda()
