@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "inv_norm.cuh"
 #include "tv_body.cuh"
 
 namespace cslsm {

@@ -9,7 +9,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 SRC = r"""
-#include "tv_body.cuh"
+#include "inv_norm.cuh"
 using namespace cslsm;
 __global__ void check_kernel(const float *s, size_t n, unsigned *bad, float *first)
 {
