@@ -623,7 +623,7 @@ def run_tvz(args) -> None:
     b_d = b_h.to(dev)
     v_d = torch.empty((w.Z, w.H, w.W), dtype=torch.float32, device=dev)
     plan = cs.Plan(w.H, w.W, 1, w.Z, masks_d)
-    cs.set_autotune(1)  # the warm-up steps time the TV kernel variants once
+    cs.set_autotune(1)  # the warm-up steps time the sweep's tilings once
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
     stream = torch.cuda.current_stream()
 
@@ -837,15 +837,19 @@ def run_secondary(args) -> None:
                    dominant_share=ms_dom / sum(ms), psnr_db=oracle.psnr(v.double().cpu().numpy(),
                                                                         data["x"]))
         if den == "tikhonov":
-            R = wk.Z
-            # the streaming model of the iterations one launch runs (all of them when the
-            # solve keeps its pixel columns on chip: then `frac` compares, it does not bound)
-            bytes_launch = vox * (16.0 + 8.0 / R) * iters * steps / n_dom
+            # one launch = the whole solve, each pixel column on chip: bound by its FP32
+            # operations; it moves the pattern words, b and v^K.  The streaming model (u, d
+            # read and written by every iteration) stands apart, it is no traffic here.
             avg = ms_dom / n_dom / 1e3
-            out["roofline"] = {"bound": "hbm", "kernel": dom, "achieved": bytes_launch / avg / 1e9,
-                               "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                               "frac": bytes_launch / avg / 1e9 / peaks["hbm_gbs"],
-                               "bytes_per_launch": bytes_launch, "avg_launch_us": avg * 1e6}
+            fl = vox * iters * (9.0 if gam > 0.0 else 6.0) * steps / n_dom
+            moved = 4.0 * vox + 8.0 * wk.H * wk.W
+            out["roofline"] = {"bound": "alu", "kernel": dom, "achieved": fl / avg / 1e12,
+                               "peak": alu_peak_tflops(2070.0), "unit": "TFLOP/s",
+                               "frac": fl / avg / 1e12 / alu_peak_tflops(2070.0),
+                               "bytes_per_launch": moved, "hbm_GBs": moved / avg / 1e9,
+                               "avg_launch_us": avg * 1e6,
+                               "streaming_model_GBs": vox * (16.0 + 8.0 / wk.Z) * iters * steps
+                               / n_dom / avg / 1e9}
         elif den == "tv" and dom == DOMINANT:
             # one launch = the whole solve; the streaming model of the prox as the
             # headline counts it, against the measured HBM copy bandwidth

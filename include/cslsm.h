@@ -417,15 +417,17 @@ int cslsm_abi_version(void);
 
 /* TV prox tile shapes (process-wide setting).  The TV kernel comes in four
  * variants (column chunks x row bands) with a tile shape chosen per launch
- * geometry; it runs where the phase launches (see cslsm_set_tv_route) do not:
- * under stream capture before their exchange exists, beyond its size, and when
- * forced.  mode 0 (default): shapes from a cost model of the work per SM.
+ * geometry; it runs where the phase launches (see cslsm_set_tv_route) do not: in
+ * cslsm_denoise without scratch, under stream capture before a plan's exchange
+ * exists, beyond its size, and when forced.  mode 0 (default): shapes from a cost model of the work per SM.
  * mode 1: on the first launch of each (device, H, W, steps, slices) key that
  * is not being captured into a CUDA graph, time every variant on the actual
  * launch (three runs each; the prox is idempotent, so this only costs time)
  * with a synchronisation of the stream, and keep the fastest for later
  * launches.  modes 2..5: force variant mode - 2 (for tests).  Changing the
- * mode clears the kept choices. */
+ * mode clears the kept choices.  Mode 1 also times the z sweep's tilings
+ * (cslsm_zsweep_config) and a batch's steps per phase (cslsm_batch_create); the
+ * phase launches are not timed, their shape is a model's in modes 0 and 1. */
 cslsm_status cslsm_set_autotune(int mode);
 
 /* The shape a tile-kernel prox launch of this geometry would use now (on the
@@ -437,8 +439,8 @@ cslsm_status cslsm_tv_shape(int H, int W, int steps, int nslices, int *shape4);
  * of cslsm_admm_solve (the Gauss-Seidel sweep over slices of Sec. III-C) runs
  * in ONE cooperative launch per ADMM iteration (enable = 1, the default):
  * every CTA owns one tile of every slice and trades the dual field of its
- * tile with its neighbours every few Chambolle steps.  enable = 0 runs one
- * tile-kernel launch per slice instead; the two give bit-identical results.
+ * tile with its neighbours every few Chambolle steps.  enable = 0 runs
+ * each slice's prox by itself instead; the two give bit-identical results.
  * tiling < 0: the tiling is chosen per (device, H, W, Z, steps, storage) key
  * by a cost model, or under cslsm_set_autotune(1) by timing every tiling once
  * on scratch copies of u and d (outside stream capture; synchronises the
@@ -469,8 +471,8 @@ unsigned long long cslsm_launch_count(void);
  * each kernel is bracketed by two CUDA events recorded on its stream (the
  * events add a little GPU time of their own); 0 switches sampling off.
  * Kernel names: "pack_masks", "forward", "adjoint", "xupdate_w",
- * "tikhonov_iter", "tikhonov_prox", "tv_tile", "psnr_partials",
- * "reduce_finish", "bm3d_prep", "bm3d_match", "bm3d_filter", "bm3d_finish",
+ * "tikhonov_iter" (an iteration or a whole solve), "tikhonov_prox", "tv_tile" (a TV
+ * prox or a phase of it), "psnr_partials", "reduce_finish", "bm3d_prep", "bm3d_match", "bm3d_filter", "bm3d_finish",
  * "batch_persistent", "unrolled", "tvz_sweep", "ssim3d". */
 cslsm_status cslsm_timing_enable(int period);
 

@@ -416,13 +416,16 @@ def bm3d_stage_groups(stage: int, noisy: torch.Tensor, sigma: float,
 
 
 def set_autotune(mode: int) -> None:
-    """TV tile shapes: 0 cost model, 1 timed autotuning, 2..5 force a variant."""
+    """0 choices by cost models and rules; 1 timed: the z sweep's tiling, a batch's steps per
+    phase and, where the whole prox runs in one launch, the TV tiles; 2..5 force a variant
+    of those tiles for every slice-independent prox."""
     _check(lib().cslsm_set_autotune(int(mode)), "cslsm_set_autotune")
 
 
 def set_tv_route(mode: int) -> None:
-    """Slice-independent TV solves: 0 auto (a one-item persistent batch for large
-    volumes), 1 per-launch tiles, 2 always the batch; the same bits either way."""
+    """Slice-independent TV solves: 0 auto (launches of a few steps each; a one-item
+    persistent batch for large volumes with BF16 or FP16 state), 1 launches, 2 always the
+    batch; the same bits either way."""
     _check(lib().cslsm_set_tv_route(int(mode)), "cslsm_set_tv_route")
 
 
@@ -433,7 +436,8 @@ def set_batch_steps_per_phase(k: int) -> None:
 
 
 def tv_shape(H: int, W: int, steps: int, nslices: int) -> dict:
-    """The TV kernel variant and tile shape a launch of this geometry uses now."""
+    """The variant and tile shape that a prox of this geometry uses now where it runs in
+    one launch (forced, captured before the exchange exists, or without scratch)."""
     buf = (ctypes.c_int * 4)()
     _check(lib().cslsm_tv_shape(int(H), int(W), int(steps), int(nslices), buf),
            "cslsm_tv_shape")
@@ -581,7 +585,7 @@ def unrolled_admm(logits: torch.Tensor, b: torch.Tensor, rho: torch.Tensor, lam:
                   keep_duals: bool = False) -> torch.Tensor:
     """Differentiable v^K of the unrolled PnP-ADMM with relaxed masks sigmoid(logits)
     [B,Z,H,W] and Huber-TV + z prior; b [B,H,W]; rho, lam, gamma 0-dim tensors.
-    keep_duals: the backward keeps the dual iterates of a checkpoint segment
+    keep_duals: the backward keeps the dual steps of a checkpoint segment
     instead of recomputing them per slice (more device memory, same gradients)."""
     cfg = dict(iters=iters, tv_steps=tv_steps, tv_tau=tv_tau, huber_eps=huber_eps,
                ckpt_every=ckpt_every, keep_duals=keep_duals)

@@ -138,9 +138,10 @@ struct TvSlices {
     int T;               // Chambolle steps
     const int *stop = nullptr;  // device flag of a tolerance-stopped solve: skip when set
 };
-// Chambolle TV prox of every listed slice.  Uses the plan-provided dual
-// buffers pbuf (4 * nslices * H * W floats) only when T exceeds the largest
-// step count one launch covers; pbuf may be nullptr otherwise.
+// Chambolle TV prox of every listed slice: in launches of a few steps each, whose
+// exchange of the dual field is pbuf (tv_pbuf_floats); without it, or with a smaller one,
+// in one launch of whole-prox tiles, which needs pbuf too beyond
+// tv_max_steps_per_launch() steps.  pbuf may be nullptr otherwise.
 cslsm_status tv_prox_slices(const TvSlices &a, float *pbuf, size_t pbuf_floats, cudaStream_t s);
 // Floats of the dual-field exchange that a prox of this geometry wants (on the current
 // device; more than tv_max_steps_per_launch() steps need it, others run without).
@@ -149,9 +150,9 @@ size_t tv_pbuf_floats(int H, int W, int T, int nslices);
 // slices fit a grid.
 bool tv_phases_fit(int H, int W, int nslices);
 int tv_max_steps_per_launch();
-// 0: tile shapes from the cost model; 1: time the kernel variants on the first
-// launch of every shape key (outside stream capture) and keep the fastest;
-// 2 + k: force variant k (tests).
+// Whole-prox tiles: 0: shapes from the cost model; 1: time the kernel variants on the
+// first launch of every shape key (outside stream capture) and keep the fastest; 2 + k:
+// force variant k (tests; the phase launches are then left out).
 void tv_set_mode(int mode);
 int tv_get_mode();
 // The shape (variant, TH, TW, RH) a launch of this geometry would use now.
