@@ -642,6 +642,7 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
     for (int q = 0; q < kRing - 1; ++q) ring.fetch(q, q < groups);
     float *Hb = a.Hb + bi * HW, *Hbar = a.Hbar + bi * HW;
     float2 b1[RPW], b2[RPW], sq[RPW], hb[RPW];
+    __shared__ Pair32 s_first[NW * 32];  // the thread's -<ubar, div p^T>, over the steps
     Pair32 sum[3] = {};  // theta, and in the last phase rho, gamma
     if (a.Pin) {
         const float *P1 = a.Pin + (size_t)bi * 2 * HW, *P2 = P1 + HW;
@@ -684,7 +685,7 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
             b2[i] = mul2(sub2(make_float2(u[i].y, ur), u[i]), splat(a.theta));
             t.mask(i, b1[i], b2[i]);
         }
-        sum[0] = part.total();
+        s_first[threadIdx.x] = part.total();
     }
 #pragma unroll
     for (int i = 0; i < RPW; ++i) sq[i] = make_float2(0.f, 0.f);
@@ -713,6 +714,7 @@ __global__ void __launch_bounds__(NW * 32, RPW == 2 ? 2 : 1) huber_bwd_kernel(co
     }
     const Pair32 tq = tqs.total();
     // kappa = eps / theta: d/dtheta of -tau kappa <abar, p>
+    if (!a.Pin) sum[0] = s_first[threadIdx.x];
     sum[0].add_scaled(tk, tk_err, a.kfac);
     sum[0].add_scaled(tq.hi, tq.lo, a.it2);
     if (a.Pout) {
