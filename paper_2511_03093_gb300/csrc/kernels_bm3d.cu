@@ -104,8 +104,8 @@ __global__ void bm3d_prep_kernel(const S *__restrict__ src, const S *__restrict_
 // 31.9 / 39.6, 1 x 512 x 512 78 / 113; one warp per reference took 17.3, 32.9, 53.9, 155.
 //   Measured, 4 slices of 512 x 512 (115,600 references): hard 0.683 -> 0.272 ms,
 // Wiener 0.659 -> 0.287 ms against one warp per reference on dp4a with sorted
-// insertion; 1,470 warp instructions a reference (5,530), bound by issue (57 %, integer
-// pipe 42 %, tensor pipe 29 %).
+// insertion; 1,420 warp instructions a reference (5,530), bound by issue (61 %, integer
+// pipe 42 %, tensor pipe 32 %).
 // mma.sync rather than tcgen05: every product goes through the ALU in the registers
 // where mma.sync leaves it, and the tensor pipe is not the limit.
 constexpr int kMSpan = 48;        // candidate rows / columns of a warp's 4 x 4 references

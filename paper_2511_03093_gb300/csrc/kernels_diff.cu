@@ -206,7 +206,7 @@ __global__ void ux_bwd_kernel(const float *__restrict__ U, const float *__restri
 // the slots, 43 us for 7 steps of 8 x 512 x 512), the reverse too (73 %, 86 us for
 // 5), and one small slice by the latency of a step and of a launch.  Forward +
 // backward, 10 iterations: 16 x 256 x 256 75.8 -> 17.8 ms; 8 x 16 x 512 x 512 with
-// the duals kept 242.5 -> 116.7 ms.
+// the duals kept 242.5 -> 117.7 ms.
 //
 //   forward  first phase: h = (rho w_n + gamma (u_{n-1} + u_{n+1})) / (rho + 2
 //            gamma) on the region (kept for the later phases and the reverse
